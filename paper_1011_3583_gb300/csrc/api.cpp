@@ -56,7 +56,7 @@ rearr_status rearr_permute(void *dst, const void *src, size_t elem_bytes, int ra
     std::string err;
     rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err);
     if (st != REARR_OK) return fail(st, "rearr_permute: " + err);
-    cudaError_t e = launch_single(pl.op, nullptr, reinterpret_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_permute(pl, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "rearr_permute launch");
     return REARR_OK;
 }
@@ -69,7 +69,7 @@ rearr_status rearr_reorder_nm(void *dst, const void *src, size_t elem_bytes, int
     std::string err;
     rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err);
     if (st != REARR_OK) return fail(st, "rearr_reorder_nm: " + err);
-    cudaError_t e = launch_single(pl.op, nullptr, reinterpret_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_permute(pl, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "rearr_reorder_nm launch");
     return REARR_OK;
 }

@@ -5,6 +5,7 @@
 
 #include <atomic>
 
+#include "plan.h"
 #include "rearr_internal.h"
 
 namespace rearr {
@@ -15,6 +16,14 @@ extern std::atomic<uint64_t> g_launches;
 // Launch the one-op kernel of `op` on stream s.  planes_all holds the k plane
 // pointers of an interlace / de-interlace (ignored otherwise).
 cudaError_t launch_single(const OpDesc &op, char *const *planes_all, cudaStream_t s);
+
+// A planned permute or N-to-M box as a single call: its span copy if it has
+// one (k_span.cu), else the kernel of its op.
+cudaError_t launch_span(const SpanDesc &d, cudaStream_t s);
+inline cudaError_t launch_permute(const PermPlan &pl, cudaStream_t s)
+{
+    return pl.use_span ? launch_span(pl.span, s) : launch_single(pl.op, nullptr, s);
+}
 
 // The L2-resident bucketed reorder (k_reorder_l2.cu) of a gather op with l2 set.
 cudaError_t launch_reorder_l2(const OpDesc &op, cudaStream_t s);

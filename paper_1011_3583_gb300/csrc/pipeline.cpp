@@ -303,7 +303,7 @@ rearr_status rearr_pipeline_permute(rearr_pipeline *pipe, void *dst, const void 
                       auto pl = std::make_shared<PermPlan>();
                       rearr_status st = plan_permute(l.out[0], l.in[0], elem_bytes, rank, dims, perm, *pl, err);
                       cls = pl->info.kind == REARR_KIND_NOOP ? uint32_t(OC_COPY) : pl->op.cls;
-                      go = [pl](cudaStream_t s) { return launch_single(pl->op, nullptr, s); };
+                      go = [pl](cudaStream_t s) { return launch_permute(*pl, s); };
                       return st;
                   });
 }
@@ -339,7 +339,7 @@ rearr_status rearr_pipeline_reorder_nm(rearr_pipeline *pipe, void *dst, const vo
                       auto pl = std::make_shared<PermPlan>();
                       rearr_status st = plan_reorder_nm(l.out[0], l.in[0], elem_bytes, rank_in, dims, rank_out,
                                                         order, base, range, *pl, err);
-                      go = [pl](cudaStream_t s) { return launch_single(pl->op, nullptr, s); };
+                      go = [pl](cudaStream_t s) { return launch_permute(*pl, s); };
                       return st;
                   });
 }

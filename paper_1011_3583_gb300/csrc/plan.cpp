@@ -31,6 +31,7 @@ constexpr int64_t kRunMinBytes = 128;     // cells this large are copied as runs
 constexpr int64_t kRunUnitBytes = 32768;  // payload of one runs work unit
 constexpr uint64_t kReorderL2MinBytes = uint64_t(128) << 20;  // reorder sources this large use L2 passes
 constexpr uint64_t kMaxUnits = 0xFFFFFFFFull;
+constexpr uint64_t kSpanMinCells = uint64_t(3) << 18;  // smaller thin-plane ops stay strided copies
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t &out)
 {
@@ -44,11 +45,6 @@ bool ranges_overlap(uintptr_t a, uint64_t na, uintptr_t b, uint64_t nb)
     if (na == 0 || nb == 0) return false;
     return a < b + nb && b < a + na;
 }
-
-struct Axis {
-    int64_t extent;
-    int64_t stride;  // input stride in bytes
-};
 
 }  // namespace
 
@@ -552,6 +548,7 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     const int W = pow2_align(da, sa, uint64_t(cell), strides_or);
     info.word_bytes = W;
     int vin = 0, vout = 0, qa = -1, qb = -1;
+    bool narrow = false;  // a fast tile that moves less than 16 bytes at a time on a side
     if (W == cell) {
         const int E = int(cell);
         // Widest legal global access on each side.  Input rows start at src
@@ -588,7 +585,8 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
         // vectorised widths the shape that fills the plane best (a widened
         // plane: the shape with the longest runs on both sides).
         TileShape shape{default_rowb(E), kTileBytes};
-        if (vin == 16 && vout == std::min(16, 4 * E)) {
+        narrow = vin < 16 || vout < std::min(16, 4 * E);
+        if (!narrow) {
             shape = (qa >= 0 || qb >= 0) ? choose_wide_shape(E, DA, DB, t.DA, t.DB) : choose_shape(E, DA, DB);
             if (shape.tbytes < kTileBytes) vout = half_tile_vout(E);
         }
@@ -668,15 +666,31 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
         info.n_tiles = int64_t(op.units);
     }
     const uint64_t n_cells = bytes / uint64_t(cell);
-    const ThinTuning thin = thin_tuning();
+    const ThinTuning thin_rule = thin_tuning();
     // (a threshold above what a tile holds means: every under-filled tile;
     // ops whose tiles are all full stay tiles)
-    const uint64_t cells_rule = std::min<uint64_t>(thin.tile_cells, uint64_t(t.TA) * t.TB);
-    const bool thin_plane = bytes < op.units * thin.tile_bytes ||
-                            (bytes <= thin.l2_bytes && n_cells < op.units * cells_rule);
+    const uint64_t cells_rule = std::min<uint64_t>(thin_rule.tile_cells, uint64_t(t.TA) * t.TB);
+    const bool thin_plane = bytes < op.units * thin_rule.tile_bytes ||
+                            (bytes <= thin_rule.l2_bytes && n_cells < op.units * cells_rule);
     if (W == cell && thin_plane && n_cells < kMaxUnits &&
         !(uint64_t(cell) <= box_max_cell_bytes() && plan_box(ax, cell, da, sa, static_cast<char *>(dst), src, op, info)))
         set_strided(W, n_cells);
+    // What a single call runs instead (the batched kernel keeps the op above).
+    // Span copies, against what else ran: tiles off the 16-byte grid
+    // (251 x 333 x 517 in order 2,0,1: 1-byte cells 112 -> 31 us, 2-byte 139 ->
+    // 52, 4-byte 150 -> 68, 8-byte 136 -> 120; with 16-byte loads an 8-byte tile
+    // is as fast: 23 against 28 us for 381 x 22 x 16 x 72 reversed in pairs),
+    // tiles less than two thirds full (32 x 16 x 4 x 3520 x 4 fp32 in order
+    // 1,0,4,2,3: 219 -> 38 us), and thin planes of 1- to 4-byte cells (2^22 x 9
+    // x 7 bytes: 344 -> 154 us).  Strided copies of 8 and 16 bytes run at the
+    // copy rate already, and small ones are over before a span copy has its
+    // tables (1479 x 381 2-byte cells: 4.7 against 5.2 us; 1001 x 999 bytes:
+    // 6.7 against 5.1).
+    if (W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
+    const bool sparse = op.cls == OC_TILE && 3 * n_cells < 2 * op.units * uint64_t(t.TA) * t.TB;
+    const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
+    if ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16)))
+        pl.use_span = plan_span(ax, cell, static_cast<char *>(dst), src, pl.span);
     return REARR_OK;
 }
 
@@ -1141,7 +1155,7 @@ bool selftest_host(std::string &err)
         err = "pow2_align";
         return false;
     }
-    return selftest_box(err);
+    return selftest_box(err) && selftest_span(err);
 }
 
 }  // namespace rearr

@@ -9,12 +9,20 @@
 
 #include "../../include/librearr.h"
 #include "rearr_internal.h"
+#include "span.h"
 
 namespace rearr {
 
+struct Axis {
+    int64_t extent;
+    int64_t stride;  // input stride in bytes
+};
+
 struct PermPlan {
     rearr_permute_info info;  // what rearr_permute_describe reports
-    OpDesc op;                // descriptor of the kernel that runs it
+    OpDesc op;                // descriptor of the body that runs it (in a batch, always this one)
+    SpanDesc span;            // the span copy a single call runs instead,
+    bool use_span;            // if there is one
 };
 
 struct InterlacePlan {
@@ -37,12 +45,19 @@ rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_
 rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, int k, size_t n,
                             size_t elem_bytes, InterlacePlan &pl, std::string &err);
 
+// Span copy of the canonical axes (output order, slowest first; input strides
+// in bytes; one E-byte word a cell): false where it does not apply.
+bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d);
+
 // A fast tile planned with the 32 KB payload re-planned with the 16 KB tile of
 // the same row length (the batched kernel holds two 16 KB tiles per CTA).
 void tile_to_single_width(OpDesc &op);
 
 // Largest power of two <= 16 dividing every argument.
 int pow2_align(uint64_t a, uint64_t b = 0, uint64_t c = 0, uint64_t d = 0);
+
+// Span plans of pseudo-random permutes run on the host against the permute.
+bool selftest_span(std::string &err);
 
 // Host self-checks of the integer helpers (fast division, alignment).
 bool selftest_host(std::string &err);

@@ -1,0 +1,96 @@
+"""Permutes off the 16-byte grid and of thin planes (span copies) on the GPU, byte for byte against the oracle, at the sizes where
+their units, words and lanes come out uneven."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests.gpu_util import DevBuf, sync, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lr():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1011_3583_gb300 import build, librearr
+    build.build()
+    librearr.load()
+    return librearr
+
+
+@pytest.fixture(scope="module")
+def orc():
+    return oracle.get()
+
+
+def check(lr, orc, e, dims, perm, src_off=0, dst_off=0):
+    n = int(np.prod(dims))
+    src = synth.random_elements(n % 1009, n, e)
+    s, d = to_dev(src, src_off), DevBuf(n * e, dst_off, fill=0x55)
+    lr.permute(d.ptr, s.ptr, e, dims, perm)
+    sync()
+    assert np.array_equal(d.download(), orc.permute(src, e, dims, perm)), (e, dims, perm, src_off, dst_off)
+
+
+# odd planes; a rank-5 op with short axes on both sides; thin planes both ways;
+# one unit with a single cell left over; output spans over several axes; a
+# unit's whole axes on both sides (no ranges)
+SPANS = [([257, 255], [1, 0]), ([1031, 1027], [1, 0]), ([61, 67, 129], [2, 0, 1]), ([5, 33, 7, 11, 63], [4, 1, 2, 0, 3]),
+         ([3, 5, 129, 517], [0, 2, 3, 1]), ([3, 129, 517, 5], [0, 3, 1, 2]), ([9973, 9, 7], [0, 2, 1]),
+         ([64 * 5 + 1, 64 * 7 + 1], [1, 0]), ([41, 23, 2, 4, 93], [1, 3, 0, 4, 2]), ([8193, 65], [1, 0]),
+         ([31, 6, 16, 42, 4], [3, 4, 0, 1, 2]), ([7, 11, 13, 17, 19, 2], [5, 3, 1, 0, 2, 4])]
+
+
+@pytest.mark.parametrize("e", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("dims,perm", SPANS)
+def test_spans(lr, orc, e, dims, perm):
+    check(lr, orc, e, dims, perm)
+
+
+@pytest.mark.parametrize("e,src_off,dst_off", [(1, 1, 0), (1, 0, 3), (1, 7, 13), (2, 2, 6), (2, 14, 0), (4, 4, 8),
+                                               (4, 12, 0), (8, 8, 8)])
+def test_spans_unaligned(lr, orc, e, src_off, dst_off):
+    """Base addresses off the grid: planes that would otherwise be 16-byte tiles."""
+    for dims, perm in (([512, 1024], [1, 0]), ([64, 96, 320], [2, 1, 0]), ([4, 3, 64, 1024], [0, 2, 3, 1])):
+        check(lr, orc, e, dims, perm, src_off, dst_off)
+
+
+def test_boxes(lr, orc):
+    """Sub-boxes: rows that are not dense in the input."""
+    g = synth.rng(7)
+    for e in (1, 2, 4):
+        dims = [37, 190, 211]
+        src = synth.random_elements(e, int(np.prod(dims)), e)
+        s = to_dev(src)
+        for order in ([2, 1, 0], [2, 0, 1], [1, 2, 0]):
+            base = [int(g.integers(0, 5)) for _ in dims]
+            rng = [d - b - int(g.integers(0, 9)) for d, b in zip(dims, base)]
+            d = DevBuf(int(np.prod([rng[a] for a in order])) * e, 0, fill=0x55)
+            lr.reorder_nm(d.ptr, s.ptr, e, dims, order, base, rng)
+            sync()
+            assert np.array_equal(d.download(), orc.reorder_nm(src, e, dims, order, base, rng)), (e, order, base, rng)
+
+
+def test_capture(lr, orc):
+    """Span copies captured in a graph and replayed on new contents."""
+    import torch
+    cases = [(1, [61, 67, 129], [2, 0, 1]), (2, [64, 3, 4096], [0, 2, 1])]
+    bufs = []
+    for e, dims, perm in cases:
+        n = int(np.prod(dims))
+        bufs.append((DevBuf(n * e, fill=0), DevBuf(n * e, fill=0)))
+    st = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        for (e, dims, perm), (s, d) in zip(cases, bufs):
+            lr.permute(d.ptr, s.ptr, e, dims, perm, torch.cuda.current_stream())
+    for seed in (1, 2):
+        srcs = [synth.random_elements(seed, int(np.prod(dims)), e) for e, dims, _ in cases]
+        for a, (s, _) in zip(srcs, bufs):
+            s.upload(a)
+        graph.replay()
+        sync()
+        for a, (e, dims, perm), (_, d) in zip(srcs, cases, bufs):
+            assert np.array_equal(d.download(), orc.permute(a, e, dims, perm)), (seed, e, dims, perm)
