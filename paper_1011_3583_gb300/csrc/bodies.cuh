@@ -745,15 +745,15 @@ __device__ __forceinline__ void deinterleave_regs(const uint32_t (&in)[K * 4], u
 
 // Element-wise tail of an interlace / de-interlace: records [r0, n).
 template <int E>
-__device__ __forceinline__ void interlace_tail(const InterlaceDesc &d, char *const *planes, uint64_t r0,
-                                               bool inter)
+__device__ __forceinline__ void interlace_tail(const InterlaceDesc &d, char *const *planes, int64_t ioff, int64_t poff,
+                                               uint64_t r0, bool inter)
 {
     const uint64_t cnt = (d.n - r0) * d.k;
     for (uint64_t f = tid_x(); f < cnt; f += kThreads) {
         const uint64_t i = r0 + f / d.k;
         const uint32_t j = uint32_t(f % d.k);
-        char *iv = d.inter + (i * d.k + j) * E;
-        char *pl = planes[j] + i * E;
+        char *iv = d.inter + ioff + (i * d.k + j) * E;
+        char *pl = planes[j] + poff + i * E;
         if (inter) stg<E>(iv, lds<E>(pl));  // plain (coherent) loads: tail is tiny
         else stg<E>(pl, lds<E>(iv));
     }
@@ -1048,7 +1048,8 @@ __device__ __forceinline__ int stage_pos(int l, int x)
 
 template <int E, int K>
 __device__ __forceinline__ void interlace_fast_body(const InterlaceDesc &d, char *const *planes, uint64_t unit,
-                                                    uint64_t n_units, unsigned char *smem)
+                                                    uint64_t n_units, unsigned char *smem, int64_t ioff = 0,
+                                                    int64_t poff = 0)
 {
     const uint64_t groups = d.n * E / 16;
     const uint64_t g0 = unit * d.unit_groups;
@@ -1061,7 +1062,7 @@ __device__ __forceinline__ void interlace_fast_body(const InterlaceDesc &d, char
             uint32_t in[K][4], out[K * 4];
 #pragma unroll
             for (int j = 0; j < K; ++j) {
-                const uint4 v = ldg_stream<16>(planes[j] + g * 16);
+                const uint4 v = ldg_stream<16>(planes[j] + poff + g * 16);
                 in[j][0] = v.x; in[j][1] = v.y; in[j][2] = v.z; in[j][3] = v.w;
             }
             interleave_regs<E, K>(in, out);
@@ -1071,7 +1072,7 @@ __device__ __forceinline__ void interlace_fast_body(const InterlaceDesc &d, char
         }
         __syncwarp();
         const uint32_t nq = uint32_t(min(uint64_t(32), g1 - gw)) * K;  // chunks of this warp's groups
-        char *o = d.inter + gw * 16 * K;
+        char *o = d.inter + ioff + gw * 16 * K;
 #pragma unroll
         for (int sidx = 0; sidx < K; ++sidx) {
             const uint32_t q = uint32_t(sidx) * 32 + lane;
@@ -1083,12 +1084,13 @@ __device__ __forceinline__ void interlace_fast_body(const InterlaceDesc &d, char
     // Every warp is done with its staging before the CTA's next body (in the
     // batched kernel another op's body) writes shared memory.
     __syncthreads();
-    if (unit == n_units - 1 && groups * 16 / E < d.n) interlace_tail<E>(d, planes, groups * 16 / E, true);
+    if (unit == n_units - 1 && groups * 16 / E < d.n) interlace_tail<E>(d, planes, ioff, poff, groups * 16 / E, true);
 }
 
 template <int E, int K>
 __device__ __forceinline__ void deinterlace_fast_body(const InterlaceDesc &d, char *const *planes, uint64_t unit,
-                                                      uint64_t n_units, unsigned char *smem)
+                                                      uint64_t n_units, unsigned char *smem, int64_t ioff = 0,
+                                                      int64_t poff = 0)
 {
     const uint64_t groups = d.n * E / 16;
     const uint64_t g0 = unit * d.unit_groups;
@@ -1097,7 +1099,7 @@ __device__ __forceinline__ void deinterlace_fast_body(const InterlaceDesc &d, ch
     uint4 *stage = reinterpret_cast<uint4 *>(smem) + warp * K * 32;
     for (uint64_t gw = g0 + uint64_t(warp) * 32; gw < g1; gw += kThreads) {
         const uint32_t nq = uint32_t(min(uint64_t(32), g1 - gw)) * K;
-        const char *src = d.inter + gw * 16 * K;
+        const char *src = d.inter + ioff + gw * 16 * K;
         uint4 v[K];
 #pragma unroll
         for (int sidx = 0; sidx < K; ++sidx) {
@@ -1122,12 +1124,12 @@ __device__ __forceinline__ void deinterlace_fast_body(const InterlaceDesc &d, ch
             deinterleave_regs<E, K>(in, out);
 #pragma unroll
             for (int j = 0; j < K; ++j)
-                stg<16>(planes[j] + g * 16, make_uint4(out[j][0], out[j][1], out[j][2], out[j][3]));
+                stg<16>(planes[j] + poff + g * 16, make_uint4(out[j][0], out[j][1], out[j][2], out[j][3]));
         }
         __syncwarp();
     }
     __syncthreads();  // staging free for the CTA's next body
-    if (unit == n_units - 1 && groups * 16 / E < d.n) interlace_tail<E>(d, planes, groups * 16 / E, false);
+    if (unit == n_units - 1 && groups * 16 / E < d.n) interlace_tail<E>(d, planes, ioff, poff, groups * 16 / E, false);
 }
 
 // Generic interlace / de-interlace: any k, any element size (c words of W

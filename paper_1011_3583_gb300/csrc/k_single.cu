@@ -102,8 +102,19 @@ __global__ void __launch_bounds__(kThreads) k_inter_fast(const __grid_constant__
     pdl_enter();
     __shared__ __align__(16) unsigned char smem[kThreads / 32 * K * 32 * 16];
     for (uint64_t u = blockIdx.x; u < n; u += gridDim.x) {
-        if constexpr (INTER) interlace_fast_body<E, K>(p.d, p.planes, u, n, smem);
-        else deinterlace_fast_body<E, K>(p.d, p.planes, u, n, smem);
+        uint64_t unit = u, units = n;
+        int64_t ioff = 0, poff = 0;
+        if (p.d.upb.d < n) {  // a batch of interlaces (units < 2^32)
+            uint32_t b, r, b0, b1;
+            fdivmod(uint32_t(u), p.d.upb, b, r);
+            fdivmod(b, p.d.b0_div, b1, b0);
+            unit = r;
+            units = p.d.upb.d;
+            ioff = int64_t(b0) * p.d.b_inter[0] + int64_t(b1) * p.d.b_inter[1];
+            poff = int64_t(b0) * p.d.b_plane[0] + int64_t(b1) * p.d.b_plane[1];
+        }
+        if constexpr (INTER) interlace_fast_body<E, K>(p.d, p.planes, unit, units, smem, ioff, poff);
+        else deinterlace_fast_body<E, K>(p.d, p.planes, unit, units, smem, ioff, poff);
     }
 }
 

@@ -676,6 +676,11 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
         !(uint64_t(cell) <= box_max_cell_bytes() && plan_box(ax, cell, da, sa, static_cast<char *>(dst), src, op, info)))
         set_strided(W, n_cells);
     // What a single call runs instead (the batched kernel keeps the op above).
+    // Interlaces of a few planes, on 16-byte boundaries: the warp-staged
+    // kernel moves 16 bytes at a time on every side.  32 x 3 x 1024^2 NCHW ->
+    // NHWC, against the strided copy: 1-byte cells 106 -> 32 us, 2-byte 111 ->
+    // 61, 4-byte 138 -> 119; 2^20-odd cells of 8 bytes in short planes gain
+    // nothing below kSpanMinCells.
     // Span copies, against what else ran: tiles off the 16-byte grid
     // (251 x 333 x 517 in order 2,0,1: 1-byte cells 112 -> 31 us, 2-byte 139 ->
     // 52, 4-byte 150 -> 68, 8-byte 136 -> 120; with 16-byte loads an 8-byte tile
@@ -689,9 +694,73 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     if (W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
     const bool sparse = op.cls == OC_TILE && 3 * n_cells < 2 * op.units * uint64_t(t.TA) * t.TB;
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
-    if ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16)))
+    pl.use_planes = (thin || narrow || sparse) &&
+                    plan_planes(ax, cell, static_cast<char *>(dst), src, pl.planes_op, pl.planes);
+    if (!pl.use_planes && ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16))))
         pl.use_span = plan_span(ax, cell, static_cast<char *>(dst), src, pl.span);
     return REARR_OK;
+}
+
+// Interlace: the output's fastest axis steps over k planes that are dense in
+// the input along the axis before it.  De-interlace: the mirror image, k cells
+// dense in the input, spread over k output planes dense along the output's
+// fastest axis.  The other axes (after collapsing, at most two) are a batch.
+// k_inter_fast moves 16-byte groups on both sides, so everything has to lie on
+// 16-byte boundaries, and a plane be long enough for a warp's 32 groups.
+bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op,
+                 char *(&planes)[kInlineK])
+{
+    const int R = int(ax.size());
+    int64_t os[kMaxRank];
+    os[R - 1] = E;
+    for (int i = R - 2; i >= 0; --i) os[i] = os[i + 1] * ax[i + 1].extent;
+    int ik = -1, ip = -1;  // the axis over planes, the axis along them
+    const bool inter = ax[R - 1].extent <= kInlineK && ax[R - 2].stride == E;
+    if (inter) {
+        ik = R - 1;
+        ip = R - 2;
+    } else {
+        for (int i = 0; i < R - 1; ++i)
+            if (ax[i].stride == E && ax[i].extent <= kInlineK && ax[R - 1].stride == E * ax[i].extent) ik = i;
+        if (ik < 0) return false;
+        ip = R - 1;
+    }
+    if (R > 4) return false;
+    const int64_t k = ax[ik].extent, n = ax[ip].extent;
+    const int64_t plane = inter ? ax[ik].stride : os[ik];
+    if (n * E < 512 || (n * E) % 16 != 0) return false;
+    std::memset(&op, 0, sizeof(op));
+    InterlaceDesc &d = op.inter;
+    uint64_t align = uint64_t(uintptr_t(dst)) | uint64_t(uintptr_t(src)) | uint64_t(plane), batch = 1;
+    int nb = 0;
+    for (int i = R - 1; i >= 0; --i) {
+        if (i == ik || i == ip) continue;
+        d.b_inter[nb] = inter ? os[i] : ax[i].stride;
+        d.b_plane[nb] = inter ? ax[i].stride : os[i];
+        align |= uint64_t(os[i]) | uint64_t(ax[i].stride);
+        if (nb == 0) d.b0_div = make_fastdiv(uint32_t(ax[i].extent));
+        batch *= uint64_t(ax[i].extent);
+        ++nb;
+    }
+    if (nb == 0) d.b0_div = make_fastdiv(1);
+    if (align % 16 != 0) return false;
+    op.cls = inter ? OC_INTERLACE : OC_DEINTERLACE;
+    op.word = uint32_t(E);
+    d.inter = inter ? dst : const_cast<char *>(src);
+    for (int j = 0; j < kInlineK; ++j)
+        planes[j] = d.planes[j] = j < k ? (inter ? const_cast<char *>(src) : dst) + j * plane : nullptr;
+    d.n = uint64_t(n);
+    d.k = uint32_t(k);
+    d.c = 1;
+    d.elem_bytes = uint32_t(E);
+    d.fast = 1;
+    const uint64_t groups = uint64_t(n) * E / 16;
+    d.unit_groups = uint64_t(kThreads) * 4;
+    const uint64_t upb = (groups + d.unit_groups - 1) / d.unit_groups;
+    if (upb * batch >= kMaxUnits) return false;
+    d.upb = make_fastdiv(uint32_t(upb));
+    op.units = upb * batch;
+    return true;
 }
 
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank, const int64_t *dims,
@@ -893,6 +962,8 @@ rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, i
         d.c = 1;
         d.unit_groups = uint64_t(kThreads) * 4;
         op.units = std::max<uint64_t>(1, (groups + d.unit_groups - 1) / d.unit_groups);
+        d.upb = make_fastdiv(0xFFFFFFFFu);
+        d.b0_div = make_fastdiv(1);
     } else {
         const int W = pow2_align(align_or, elem_bytes);
         op.word = uint32_t(W);

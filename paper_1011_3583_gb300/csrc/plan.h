@@ -21,8 +21,12 @@ struct Axis {
 struct PermPlan {
     rearr_permute_info info;  // what rearr_permute_describe reports
     OpDesc op;                // descriptor of the body that runs it (in a batch, always this one)
-    SpanDesc span;            // the span copy a single call runs instead,
-    bool use_span;            // if there is one
+    // What a single call runs instead, if there is one: interlaces of a few
+    // planes, or a span copy.
+    bool use_planes, use_span;
+    OpDesc planes_op;
+    char *planes[kInlineK];
+    SpanDesc span;
 };
 
 struct InterlacePlan {
@@ -44,6 +48,11 @@ rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_
                           bool scatter = false);
 rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, int k, size_t n,
                             size_t elem_bytes, InterlacePlan &pl, std::string &err);
+
+// A permute of the canonical axes as a batch of interlaces or de-interlaces
+// (false: it is none, or not on 16-byte boundaries).
+bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op,
+                 char *(&planes)[kInlineK]);
 
 // Span copy of the canonical axes (output order, slowest first; input strides
 // in bytes; one E-byte word a cell): false where it does not apply.

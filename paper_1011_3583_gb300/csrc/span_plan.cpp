@@ -337,6 +337,29 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, std::s
     return true;
 }
 
+// Host run of interlaces planned for a permute: every cell of every plane.
+static bool planes_emulate(const OpDesc &op, char *const *planes, char *dst0, size_t dst_bytes, std::string &err)
+{
+    const InterlaceDesc &d = op.inter;
+    const int E = int(d.elem_bytes);
+    const uint64_t upb = d.upb.d, groups = d.n * E / 16;
+    if (d.n * E % 16 != 0 || upb * d.unit_groups < groups) { err = "planes: units do not cover a plane"; return false; }
+    for (uint64_t b = 0; b < op.units / upb; ++b) {
+        const int64_t b0 = int64_t(b % d.b0_div.d), b1 = int64_t(b / d.b0_div.d);
+        char *iv = d.inter + b0 * d.b_inter[0] + b1 * d.b_inter[1];
+        const int64_t poff = b0 * d.b_plane[0] + b1 * d.b_plane[1];
+        for (uint32_t j = 0; j < d.k; ++j)
+            for (uint64_t i = 0; i < d.n; ++i) {
+                char *c = iv + (i * d.k + j) * E, *pl = planes[j] + poff + i * E;
+                char *to = op.cls == OC_INTERLACE ? c : pl;
+                if (i == 0 && (uintptr_t(iv) % 16 || uintptr_t(pl) % 16)) { err = "planes: off the 16-byte grid"; return false; }
+                if (to < dst0 || to + E > dst0 + dst_bytes) { err = "planes: store outside the destination"; return false; }
+                std::memcpy(to, op.cls == OC_INTERLACE ? pl : c, E);
+            }
+    }
+    return true;
+}
+
 bool selftest_span(std::string &err)
 {
     uint64_t x = 0x9E3779B97F4A7C15ull;
@@ -344,8 +367,8 @@ bool selftest_span(std::string &err)
         x ^= x << 13; x ^= x >> 7; x ^= x << 17;
         return x % n;
     };
-    int plans = 0, partial = 0, luts = 0, shared = 0, narrow = 0;
-    for (int t = 0; t < 12000 && plans < 500; ++t) {
+    int plans = 0, partial = 0, luts = 0, shared = 0, narrow = 0, planes = 0, inter = 0;
+    for (int t = 0; t < 12000 && (plans < 500 || planes < 60); ++t) {
         const int rank = 2 + int(rnd(5));
         const int E = 1 << rnd(5);
         int64_t dims[kMaxRank];
@@ -403,6 +426,14 @@ bool selftest_span(std::string &err)
                   "-byte cells differ from the permute";
             return false;
         };
+        OpDesc op;
+        char *pl[kInlineK];
+        if (plan_planes(ax, E, dst, src, op, pl)) {
+            ++planes;
+            inter += op.cls == OC_INTERLACE;
+            std::memset(dst, 0, out_bytes);
+            if (!planes_emulate(op, pl, dst, out_bytes, err) || !same("interlaces")) return false;
+        }
         SpanDesc d;
         if (!plan_span(ax, E, dst, src, d)) continue;
         ++plans;
@@ -413,10 +444,10 @@ bool selftest_span(std::string &err)
         std::memset(dst, 0, out_bytes);
         if (!span_emulate(d, dst, out_bytes, err) || !same("the spans")) return false;
     }
-    if (plans < 300 || partial < 50 || luts < 50 || shared < 10 || narrow < 20) {
+    if (plans < 300 || partial < 50 || luts < 50 || shared < 10 || narrow < 20 || inter < 10 || planes - inter < 10) {
         err = "span self-test planned " + std::to_string(plans) + " copies (" + std::to_string(partial) + " partial, " +
               std::to_string(luts) + " of several axes, " + std::to_string(shared) + " sharing a range, " +
-              std::to_string(narrow) + " in narrow copies)";
+              std::to_string(narrow) + " in narrow copies) and " + std::to_string(planes) + " interlaces";
         return false;
     }
     return true;

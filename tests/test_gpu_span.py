@@ -1,4 +1,5 @@
-"""Permutes off the 16-byte grid and of thin planes (span copies) on the GPU, byte for byte against the oracle, at the sizes where
+"""Permutes off the 16-byte grid and of thin planes (span copies, interlaces of
+a few planes) on the GPU, byte for byte against the oracle, at the sizes where
 their units, words and lanes come out uneven."""
 import numpy as np
 import pytest
@@ -57,6 +58,20 @@ def test_spans_unaligned(lr, orc, e, src_off, dst_off):
         check(lr, orc, e, dims, perm, src_off, dst_off)
 
 
+# planes of exactly a warp's 512 bytes, one group past a unit, two batch axes,
+# k of every staging form
+@pytest.mark.parametrize("e", [1, 2, 4, 8])
+@pytest.mark.parametrize("k", [2, 3, 5, 6, 8])
+def test_planes(lr, orc, e, k):
+    for batch, p in (([37], 16448 // e), ([1201], 1024 // e), ([3, 5], 65552 // e)):
+        if len(batch) == 1:
+            check(lr, orc, e, batch + [k, p], [0, 2, 1])
+            check(lr, orc, e, batch + [p, k], [0, 2, 1])
+        else:  # the batch axes change places, so they stay two
+            check(lr, orc, e, [batch[0], batch[1], k, p], [1, 0, 3, 2])
+            check(lr, orc, e, [batch[0], batch[1], p, k], [1, 0, 3, 2])
+
+
 def test_boxes(lr, orc):
     """Sub-boxes: rows that are not dense in the input."""
     g = synth.rng(7)
@@ -74,7 +89,7 @@ def test_boxes(lr, orc):
 
 
 def test_capture(lr, orc):
-    """Span copies captured in a graph and replayed on new contents."""
+    """A span copy and planes captured in a graph and replayed on new contents."""
     import torch
     cases = [(1, [61, 67, 129], [2, 0, 1]), (2, [64, 3, 4096], [0, 2, 1])]
     bufs = []
