@@ -31,6 +31,7 @@ constexpr int64_t kRunMinBytes = 128;     // cells this large are copied as runs
 constexpr int64_t kRunUnitBytes = 32768;  // payload of one runs work unit
 constexpr uint64_t kReorderL2MinBytes = uint64_t(128) << 20;  // reorder sources this large use L2 passes
 constexpr uint64_t kMaxUnits = 0xFFFFFFFFull;
+constexpr uint64_t kGatherStepMax = uint64_t(1) << 23;  // index sequences cut into single steps
 constexpr uint64_t kSpanMinCells = uint64_t(3) << 18;  // smaller thin-plane ops stay strided copies
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t &out)
@@ -897,7 +898,13 @@ rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_
     // the contiguous side (dst of a gather, src of a scatter) in groups of 4
     const uintptr_t contiguous = scatter ? sa : da;
     g.vec = (g.c == 1 && idx_bytes == 4 && ia % 16 == 0 && contiguous % uint64_t(std::min(16, 4 * W)) == 0) ? 1u : 0u;
-    g.unit_elems = g.vec ? uint32_t(kThreads) * 32 : uint32_t(kThreads) * 16;
+    // Units of one step of the body (four elements per thread) up to
+    // kGatherStepMax elements, of two beyond: with eight steps a unit, 3M
+    // elements were 367 CTAs for 152 SMs.  3,000,017 x 8 B random gather 23.9
+    // -> 20.5 us, 4M x 16 B 57 -> 42, 65,536 x 4 B 5.1 -> 3.5, scatter of
+    // 3,000,017 x 4 B 19.8 -> 16.4; at 16M x 4 B one step 78.0, two 75.5,
+    // four 76.6, eight 78.0 us.
+    g.unit_elems = uint32_t(kThreads) * (n <= kGatherStepMax ? 4 : 8);
     op.units = (uint64_t(n) + g.unit_elems - 1) / g.unit_elems;
     // Sources much larger than the L2 go through the bucketed passes (which
     // fall back to this direct gather on the device if the indices turn out
