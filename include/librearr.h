@@ -283,7 +283,7 @@ rearr_status rearr_inject_wait_timeout(int n_launches);
 
 /* ---------------------------------------------------------------------------
  * Batched execution.  The paper has no batching; these calls run many of the
- * operations above in one persistent kernel launch driven by a device-side
+ * operations above in one persistent kernel launch (up to three) driven by a device-side
  * tile work list, captured once in a CUDA graph and replayed.
  *
  *   rearr_plan_create    : new empty plan (host object).
@@ -294,8 +294,10 @@ rearr_status rearr_inject_wait_timeout(int n_launches);
  *   rearr_plan_finalize  : builds the work list, uploads it (one device
  *                          allocation owned by the plan), picks tile shapes from
  *                          the tuning table and captures the launch in a CUDA
- *                          graph on `stream`.  No op can be added afterwards
- *                          (REARR_EBUSY).
+ *                          graph on `stream`.  A large plan's index gathers and
+ *                          scatters and its thin-plane permutes get a persistent
+ *                          kernel each beside the others'.  No op can be added
+ *                          afterwards (REARR_EBUSY).
  *   rearr_batch          : replays the captured graph on `stream`; every op of
  *                          the plan is computed exactly as its single call
  *                          would compute it.  Replays on one stream are ordered;

@@ -246,6 +246,47 @@ __global__ void __launch_bounds__(kThreads, 4) k_batch(const OpDesc *__restrict_
     }
 }
 
+// The index gathers and scatters of a captured batch, in a kernel without
+// shared memory: the SM's whole L1 is theirs (their random reads live on its
+// hits; k_batch's 128 KB of shared memory per SM leave half of it).  683
+// reorders of the 2048-op mix: 1657 us in k_batch; here 1389, 1353, 1402 us
+// at 6, 5, 4 CTAs per SM (grabs of four units of 2048 elements; 1459 at one,
+// 1733 at eight).
+__global__ void __launch_bounds__(kThreads, 5) k_batch_gather(const OpDesc *__restrict__ ops,
+                                                                       const uint64_t *__restrict__ prefix, int n_ops,
+                                                                       unsigned long long *counter, uint32_t grab)
+{
+    __shared__ unsigned long long s_start;
+    const uint64_t total = prefix[n_ops];
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_start = atomicAdd(counter, (unsigned long long)grab);
+        __syncthreads();
+        const uint64_t start = s_start;
+        if (start >= total) break;
+        const uint64_t end = min(total, start + grab);
+        int lo = 0, hi = n_ops - 1;  // last op with prefix[lo] <= start
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (prefix[mid] <= start) lo = mid;
+            else hi = mid - 1;
+        }
+        for (uint64_t t = start; t < end; ++lo) {
+            const uint64_t base = prefix[lo], seg_end = min(end, prefix[lo + 1]);
+            const OpDesc &op = ops[lo];
+            for (; t < seg_end; ++t) {
+                switch (op.word) {
+                    case 1: gather_body<1>(op.gather, t - base); break;
+                    case 2: gather_body<2>(op.gather, t - base); break;
+                    case 4: gather_body<4>(op.gather, t - base); break;
+                    case 8: gather_body<8>(op.gather, t - base); break;
+                    default: gather_body<16>(op.gather, t - base); break;
+                }
+            }
+        }
+    }
+}
+
 }  // namespace rearr
 
 // ---------------------------------------------------------------------------
@@ -256,6 +297,8 @@ using namespace rearr;
 struct rearr_plan {
     std::vector<OpDesc> ops;
     std::vector<std::vector<char *>> plane_lists;  // per op (empty unless k > kInlineK)
+    std::vector<SpanDesc> spans;       // span copies the captured batch runs in place of their ops
+    std::vector<int> span_of;          // per op, until finalize orders them: index into spans, or -1
     bool finalized = false;
     void *dev = nullptr;               // one allocation: ops | prefix | plane arrays | counter
     OpDesc *d_ops = nullptr;
@@ -267,15 +310,23 @@ struct rearr_plan {
     int n_launch_ops = 0;              // ops with at least one unit
     uint32_t grab = 1;
     int grid = 0;
+    int kernels = 0;                   // kernels of a replay
 };
 
-static rearr_status add_op(rearr_plan *p, const OpDesc &op_in, std::vector<char *> planes = {})
+constexpr uint64_t kSplitUnits = 64;
+
+namespace rearr { static int resident_ctas_current_device(); }
+
+static rearr_status add_op(rearr_plan *p, const OpDesc &op_in, std::vector<char *> planes = {},
+                           const SpanDesc *span = nullptr)
 {
     if (op_in.units == 0) return REARR_OK;
     OpDesc op = op_in;
     batch_form(op);
     p->ops.push_back(op);
     p->plane_lists.push_back(std::move(planes));
+    p->span_of.push_back(span ? int(p->spans.size()) : -1);
+    if (span) p->spans.push_back(*span);
     return REARR_OK;
 }
 
@@ -296,9 +347,9 @@ rearr_status rearr_plan_add_permute(rearr_plan *plan, void *dst, const void *src
     if (plan->finalized) return fail(REARR_EBUSY, "rearr_plan_add_permute: plan is finalized");
     PermPlan pl;
     std::string err;
-    rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err);
+    rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err, true);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_permute: " + err);
-    return add_op(plan, pl.op);
+    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
 }
 
 rearr_status rearr_plan_add_scatter(rearr_plan *plan, void *dst, const void *src, const uint32_t *idx, size_t n,
@@ -321,9 +372,9 @@ rearr_status rearr_plan_add_reorder_nm(rearr_plan *plan, void *dst, const void *
     if (plan->finalized) return fail(REARR_EBUSY, "rearr_plan_add_reorder_nm: plan is finalized");
     PermPlan pl;
     std::string err;
-    rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err);
+    rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err, true);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_reorder_nm: " + err);
-    return add_op(plan, pl.op);
+    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
 }
 
 rearr_status rearr_plan_add_reorder(rearr_plan *plan, void *dst, const void *src, const uint32_t *idx, size_t n,
@@ -372,22 +423,66 @@ rearr_status rearr_plan_finalize(rearr_plan *plan, rearr_stream_t stream)
 {
     if (!plan) return fail(REARR_EINVAL, "rearr_plan_finalize: plan is NULL");
     if (plan->finalized) return fail(REARR_EBUSY, "rearr_plan_finalize: plan is already finalized");
-    const size_t n = plan->ops.size();
     plan->finalized = true;
-    if (n == 0) return REARR_OK;
+    if (plan->ops.empty()) return REARR_OK;
+    // In a large plan permutes with a span copy go to a kernel of their own
+    // (k_batch_span: 466 thin-plane permutes of the 2048-op mix 655 us as
+    // strided copies, one L1 request a cell; 375 us), and so do index gathers
+    // and scatters (k_batch_gather).  Each kernel ramps up and drains by
+    // itself, some 40 us in all, so a plan is split from kSplitUnits work units
+    // per resident CTA up: 2048 ops 2768 -> 2256 us, 700 ops 1044 -> 886, 400
+    // ops (41,000 to 47,000 units) 651 -> 575; not split, 200 ops (23,500) 349
+    // against 335, 64 ops (6,500) 105 against 126.  The full op list, ordered,
+    // stays for rearr_batch_noalloc.
+    std::vector<OpDesc> ops, gathers;
+    std::vector<std::vector<char *>> lists;
+    uint64_t all_units = 0;
+    for (const OpDesc &op : plan->ops) all_units += op.units;
+    const bool split = all_units >= kSplitUnits * uint64_t(std::max(1, resident_ctas_current_device()));
+    if (!split) plan->spans.clear();
+    for (size_t i = 0; i < plan->ops.size(); ++i) {
+        if (split && plan->span_of[i] >= 0) continue;
+        if (split && plan->ops[i].cls == OC_GATHER) {
+            gathers.push_back(plan->ops[i]);
+            continue;
+        }
+        ops.push_back(plan->ops[i]);
+        lists.push_back(plan->plane_lists[i]);
+    }
+    std::stable_sort(gathers.begin(), gathers.end(), [](const OpDesc &a, const OpDesc &b) { return a.word < b.word; });
     order_for_batch(plan->ops, plan->plane_lists);
+    order_for_batch(ops, lists);
+    std::vector<SpanDesc> &spans = plan->spans;
+    // one body after the other, large ops first (they are the ones that could
+    // be left to the end)
+    std::stable_sort(spans.begin(), spans.end(), [](const SpanDesc &a, const SpanDesc &b) {
+        const uint32_t ka = a.E << 1 | a.lut, kb = b.E << 1 | b.lut;
+        return ka != kb ? ka < kb : a.units > b.units;
+    });
+    const size_t n = ops.size(), ns = spans.size(), ng = gathers.size();
     // Host image of the device block.
     size_t n_ptrs = 0;
-    for (auto &l : plan->plane_lists) n_ptrs += l.size();
+    for (auto &l : lists) n_ptrs += l.size();
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t off_ops = 0;
-    const size_t off_prefix = (n * sizeof(OpDesc) + 255) / 256 * 256;
-    const size_t off_planes = off_prefix + ((n + 1) * sizeof(uint64_t) + 255) / 256 * 256;
-    const size_t off_counter = off_planes + (n_ptrs * sizeof(char *) + 255) / 256 * 256;
-    const size_t total_bytes = off_counter + 256;
+    const size_t off_prefix = up(n * sizeof(OpDesc));
+    const size_t off_planes = off_prefix + up((n + 1) * sizeof(uint64_t));
+    const size_t off_counter = off_planes + up(n_ptrs * sizeof(char *));
+    const size_t off_spans = off_counter + 256;
+    const size_t off_sprefix = off_spans + up(ns * sizeof(SpanDesc));
+    const size_t off_gathers = off_sprefix + (ns ? up((ns + 1) * sizeof(uint64_t)) : 0);
+    const size_t off_gprefix = off_gathers + up(ng * sizeof(OpDesc));
+    const size_t total_bytes = off_gprefix + (ng ? up((ng + 1) * sizeof(uint64_t)) : 0);
     std::vector<unsigned char> host(total_bytes, 0);
-    std::vector<uint64_t> prefix(n + 1, 0);
-    for (size_t i = 0; i < n; ++i) prefix[i + 1] = prefix[i] + plan->ops[i].units;
+    std::vector<uint64_t> prefix(n + 1, 0), sprefix(ns + 1, 0), gprefix(ng + 1, 0);
+    for (size_t i = 0; i < ng; ++i) gprefix[i + 1] = gprefix[i] + gathers[i].units;
+    for (size_t i = 0; i < n; ++i) prefix[i + 1] = prefix[i] + ops[i].units;
     plan->total_units = prefix[n];
+    uint32_t span_smem = 0;
+    for (size_t i = 0; i < ns; ++i) {
+        sprefix[i + 1] = sprefix[i] + spans[i].units;
+        span_smem = std::max(span_smem, span_smem_bytes(spans[i]));
+    }
 
     cudaError_t e = cudaMalloc(&plan->dev, total_bytes);
     if (e != cudaSuccess) {
@@ -400,17 +495,24 @@ rearr_status rearr_plan_finalize(rearr_plan *plan, rearr_stream_t stream)
     plan->d_counter = reinterpret_cast<unsigned long long *>(base + off_counter);
     size_t pi = 0;
     for (size_t i = 0; i < n; ++i) {
-        OpDesc &op = plan->ops[i];
-        auto &l = plan->plane_lists[i];
+        auto &l = lists[i];
         if (!l.empty()) {
             char **dst = reinterpret_cast<char **>(host.data() + off_planes) + pi;
             std::memcpy(dst, l.data(), l.size() * sizeof(char *));
-            op.inter.planes_dev = reinterpret_cast<char *const *>(base + off_planes + pi * sizeof(char *));
+            ops[i].inter.planes_dev = reinterpret_cast<char *const *>(base + off_planes + pi * sizeof(char *));
             pi += l.size();
         }
     }
-    std::memcpy(host.data() + off_ops, plan->ops.data(), n * sizeof(OpDesc));
+    if (n) std::memcpy(host.data() + off_ops, ops.data(), n * sizeof(OpDesc));
     std::memcpy(host.data() + off_prefix, prefix.data(), (n + 1) * sizeof(uint64_t));
+    if (ns) {
+        std::memcpy(host.data() + off_spans, spans.data(), ns * sizeof(SpanDesc));
+        std::memcpy(host.data() + off_sprefix, sprefix.data(), (ns + 1) * sizeof(uint64_t));
+    }
+    if (ng) {
+        std::memcpy(host.data() + off_gathers, gathers.data(), ng * sizeof(OpDesc));
+        std::memcpy(host.data() + off_gprefix, gprefix.data(), (ng + 1) * sizeof(uint64_t));
+    }
     cudaStream_t us = reinterpret_cast<cudaStream_t>(stream);
     e = cudaMemcpyAsync(plan->dev, host.data(), total_bytes, cudaMemcpyHostToDevice, us);
     if (e == cudaSuccess) e = cudaStreamSynchronize(us);
@@ -430,18 +532,43 @@ rearr_status rearr_plan_finalize(rearr_plan *plan, rearr_stream_t stream)
     plan->grid = int(std::max<uint64_t>(grid, 1));
     plan->n_launch_ops = int(n);
 
-    // Capture the counter reset and the launch in a graph on a private stream.
+    // Capture the counters' reset and the launches in a graph on a private
+    // stream, one kernel after the other: side by side, the SMs kept the first
+    // one's split of L1 and shared memory for both, and the gathers' time
+    // doubled (2048 ops: 4.07 ms instead of 2.77).
     cudaStream_t cap;
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_fail(e, "rearr_plan_finalize: stream");
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaMemsetAsync(plan->d_counter, 0, sizeof(unsigned long long), cap);
-        k_batch<<<plan->grid, kThreads, 0, cap>>>(plan->d_ops, plan->d_prefix, int(n), plan->d_counter, plan->grab);
-        cudaError_t le = cudaGetLastError();
+        cudaError_t le = cudaMemsetAsync(plan->d_counter, 0, 3 * sizeof(unsigned long long), cap);
+        if (le == cudaSuccess && ng) {
+            int per = 0;
+            le = cudaFuncSetAttribute(k_batch_gather, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      cudaSharedmemCarveoutMaxL1);
+            if (le == cudaSuccess) le = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_gather, kThreads, 0);
+            const uint64_t resident = uint64_t(sms) * uint64_t(std::max(per, 1));
+            const uint32_t grab = tun.grab_for(gprefix[ng], resident);
+            const uint64_t grabs = (gprefix[ng] + grab - 1) / grab;
+            if (le == cudaSuccess) {
+                k_batch_gather<<<unsigned(std::max<uint64_t>(1, std::min(resident, grabs))), kThreads, 0, cap>>>(
+                    reinterpret_cast<const OpDesc *>(base + off_gathers),
+                    reinterpret_cast<const uint64_t *>(base + off_gprefix), int(ng), plan->d_counter + 2, grab);
+                le = cudaGetLastError();
+            }
+        }
+        if (le == cudaSuccess && n) {
+            k_batch<<<plan->grid, kThreads, 0, cap>>>(plan->d_ops, plan->d_prefix, int(n), plan->d_counter, plan->grab);
+            le = cudaGetLastError();
+        }
+        if (le == cudaSuccess && ns)
+            le = launch_batch_spans(reinterpret_cast<const SpanDesc *>(base + off_spans),
+                                    reinterpret_cast<const uint64_t *>(base + off_sprefix), int(ns), sprefix[ns],
+                                    span_smem, plan->d_counter + 1, cap);
         e = cudaStreamEndCapture(cap, &plan->graph);
         if (e == cudaSuccess && le != cudaSuccess) e = le;
     }
+    plan->kernels = (n ? 1 : 0) + (ns ? 1 : 0) + (ng ? 1 : 0);
     if (e == cudaSuccess) e = cudaGraphInstantiate(&plan->exec, plan->graph, 0);
     cudaStreamDestroy(cap);
     if (e != cudaSuccess) return cuda_fail(e, "rearr_plan_finalize: graph capture");
@@ -455,7 +582,7 @@ rearr_status rearr_batch(rearr_plan *plan, rearr_stream_t stream)
     if (!plan->exec) return REARR_OK;  // empty plan
     cudaError_t e = cudaGraphLaunch(plan->exec, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "rearr_batch: graph launch");
-    g_launches.fetch_add(1, std::memory_order_relaxed);
+    g_launches.fetch_add(uint64_t(plan->kernels), std::memory_order_relaxed);
     return REARR_OK;
 }
 

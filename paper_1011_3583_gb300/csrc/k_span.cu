@@ -16,9 +16,8 @@
 #include <algorithm>
 #include <mutex>
 
-#include "bodies.cuh"
 #include "launch.h"
-#include "span.h"
+#include "span_body.cuh"
 
 namespace rearr {
 
@@ -26,224 +25,69 @@ namespace {
 
 constexpr int kSpanCtas = 6;  // resident CTAs per SM (about 40 registers a thread; 8 spill)
 
-// Shares n_spans spans out over the CTA: `lanes` neighbouring threads walk one
-// span, kThreads / lanes spans at a time (leftover threads idle), so that an
-// instruction covers neighbouring chunks (words) of one or a few spans.
-struct SpanShare {
-    uint32_t group, lane, groups;
-    __device__ __forceinline__ explicit SpanShare(uint32_t lanes)
-    {
-        groups = kThreads / lanes;
-        group = threadIdx.x / lanes;
-        lane = threadIdx.x - group * lanes;
-        if (group >= groups) group = 0xFFFFFFFFu / 2;  // past any span
-    }
-};
-
-template <int CW>
-__device__ __forceinline__ void span_load(const SpanShare &sh, uint32_t lanes, const char *src, uint32_t rows,
-                                          uint32_t len, unsigned char *tile, const int64_t *row_in,
-                                          const uint32_t *row_sm)
-{
-    const uint32_t base = uint32_t(reinterpret_cast<uintptr_t>(src) & 15);
-    const uint32_t x0 = sh.lane * CW;
-#pragma unroll 4
-    for (uint32_t row = sh.group; row < rows; row += sh.groups) {
-        const uintptr_t g = reinterpret_cast<uintptr_t>(src) + row_in[row];
-        const uint32_t left = len + (uint32_t(g) & (CW - 1));  // bytes from the first chunk's start
-        const char *p = reinterpret_cast<const char *>(g & ~uintptr_t(CW - 1));
-        unsigned char *t = tile + ((base + row_sm[row]) & ~uint32_t(CW - 1));
-        if (x0 < left) cp_async<CW>(t + x0, p + x0);
-        for (uint32_t x = x0 + lanes * CW; x < left; x += lanes * CW) cp_async<CW>(t + x, p + x);
-    }
-}
-
-// Spans' offsets from their digits, fastest first.
-__device__ __forceinline__ void span_digits(uint32_t q, const uint32_t *ext, const int64_t *stride, const uint32_t *sms,
-                                            int64_t &off, uint32_t &sm)
-{
-    off = 0;
-    sm = 0;
-#pragma unroll
-    for (int i = 0; i < kSpanAxes; ++i) {
-        if (ext[i] == 1) continue;
-        const uint32_t n = q / ext[i], dig = q - n * ext[i];
-        q = n;
-        off += int64_t(dig) * stride[i];
-        sm += dig * sms[i];
-    }
-}
-
-// A unit's origin and what of a full unit it holds.  One thread works it out
-// for the next unit while the others store this one.
-struct SpanUnit {
-    const char *src;
-    char *dst;
-    uint32_t rows, runs, row_bytes, cells;
-};
-
-__device__ __forceinline__ void span_unit(const SpanDesc &d, uint32_t u, SpanUnit &x)
-{
-    const char *src = d.src;
-    char *dst = d.dst;
-    uint32_t rows = d.n_rows, runs = d.n_runs, row_bytes = d.row_bytes, cells = d.run_cells;
-#pragma unroll 1
-    for (int i = d.no - 1; i >= 0; --i) {
-        uint32_t dig;
-        fdivmod(u, d.udiv[i], u, dig);
-        src += int64_t(dig) * d.uin[i];
-        dst += int64_t(dig) * d.uout[i];
-        if (i == d.ua) {
-            const uint32_t k = min(d.ka, d.na - dig * d.ka);
-            row_bytes = k * d.row_bytes_a;
-            if (d.n_runs_a) runs = k * d.n_runs_a;
-            if (d.run_cells_a) cells = k * d.run_cells_a;
-        }
-        if (i == d.ub) {
-            const uint32_t k = min(d.kb, d.nb - dig * d.kb);
-            if (d.n_rows_b) rows = k * d.n_rows_b;
-            if (d.run_cells_b) cells = k * d.run_cells_b;
-        }
-    }
-    x.src = src;
-    x.dst = dst;
-    x.rows = rows;
-    x.runs = runs;
-    x.row_bytes = row_bytes;
-    x.cells = cells;
-}
-
-// Offsets of cells p .. p + V - 1 of an output span in shared memory.
-template <int V, bool LUT>
-__device__ __forceinline__ void span_offsets(const uint16_t *lut, uint32_t p, uint32_t step, uint32_t (&f)[V])
-{
-    if constexpr (!LUT) {
-        f[0] = p * step;
-#pragma unroll
-        for (int k = 1; k < V; ++k) f[k] = f[k - 1] + step;
-    } else if constexpr (V == 4) {
-        if ((p & 3) == 0) {
-            const uint2 q = lds<8>(lut + p);
-            f[0] = q.x & 0xFFFF; f[1] = q.x >> 16; f[2] = q.y & 0xFFFF; f[3] = q.y >> 16;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) f[k] = lut[p + k];
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; ++k) f[k] = lut[p + k];
-    }
-}
-
-// The word of V cells at s + f[0], s + f[1], ...
-template <int E, int V>
-__device__ __forceinline__ typename Word<E * V>::T span_word(const unsigned char *s, const uint32_t (&f)[V])
-{
-    if constexpr (V == 1) return lds<E>(s + f[0]);
-    else if constexpr (E == 2) return prmt(lds<2>(s + f[0]), lds<2>(s + f[1]), 0x5410u);
-    else return prmt(prmt(lds<1>(s + f[0]), lds<1>(s + f[1]), 0x0040u), prmt(lds<1>(s + f[2]), lds<1>(s + f[3]), 0x0040u),
-                     0x5410u);
-}
-
 template <int E, bool LUT>
 __global__ void __launch_bounds__(kThreads, kSpanCtas) k_span(const __grid_constant__ SpanDesc d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char *tile = smem;
-    int64_t *row_in = reinterpret_cast<int64_t *>(smem + d.tile_bytes);
-    int64_t *run_out = row_in + d.n_rows;
-    uint32_t *row_sm = reinterpret_cast<uint32_t *>(run_out + d.n_runs);
-    uint32_t *run_sm = row_sm + d.n_rows;
-    uint16_t *lut = reinterpret_cast<uint16_t *>(smem + span_lut_offset(d));
-    constexpr uint32_t WU = E < 4 ? 4 : E, V = WU / E;
-
-    // The tables hold for every unit; they read no global memory, so they are
-    // built before the wait for the kernel ahead on the stream.
-    for (uint32_t r = threadIdx.x; r < d.n_rows; r += kThreads)
-        span_digits(r, d.row_ext, d.row_in, d.row_sm, row_in[r], row_sm[r]);
-    for (uint32_t r = threadIdx.x; r < d.n_runs; r += kThreads)
-        span_digits(r, d.run_ext, d.run_out, d.run_sm, run_out[r], run_sm[r]);
-    if constexpr (LUT) {
-        // a thread's entries are kThreads apart: one decomposition, then steps with carries
-        uint32_t dig[kSpanAxes], step[kSpanAxes], ext[kSpanAxes], q = threadIdx.x, e = kThreads;
-#pragma unroll
-        for (int i = 0; i < kSpanAxes; ++i) {
-            ext[i] = d.ch_ext[i];
-            dig[i] = ext[i] > 1 ? q % ext[i] : 0;
-            step[i] = ext[i] > 1 ? e % ext[i] : 0;
-            q = ext[i] > 1 ? q / ext[i] : q;
-            e = ext[i] > 1 ? e / ext[i] : e;
-        }
-        for (uint32_t p = threadIdx.x; p < d.run_cells; p += kThreads) {
-            uint32_t sm = 0;
-#pragma unroll
-            for (int i = 0; i < kSpanAxes; ++i) sm += dig[i] * d.ch_sm[i];
-            lut[p] = uint16_t(sm);
-            box_advance<kSpanAxes>(dig, step, ext);
-        }
-    }
     __shared__ SpanUnit unit;
-    if (threadIdx.x == 0) span_unit(d, blockIdx.x, unit);
-    __syncthreads();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // The tables read no global memory, so they are built before the wait for
+    // the kernel ahead on the stream.
+    span_units<E, LUT>(d, blockIdx.x, d.units, gridDim.x, smem, unit, [] {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    });
+}
 
-    const uint32_t ch0 = d.ch_sm[0];
-    const SpanShare ld(d.load_lanes), st(d.store_lanes);
-    // Output spans that all start on a word boundary and take one pass: the
-    // thread's cells have the same offsets in every span of every unit.
-    uint32_t fixed[V];
-    if (d.fixed && st.lane * V + V <= d.run_cells) span_offsets<V, LUT>(lut, st.lane * V, ch0, fixed);
-    for (uint32_t u = blockIdx.x; u < d.units; u += gridDim.x) {
-        const SpanUnit x = unit;
-        if (d.chunk == 16) span_load<16>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
-        else if (d.chunk == 8) span_load<8>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
-        else span_load<4>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-        if (threadIdx.x == 0 && u + gridDim.x < d.units) span_unit(d, u + gridDim.x, unit);
+// Span copies of a batch: units of many descriptors handed out `grab` at a
+// time; each piece of a descriptor builds its tables anew, so a grab is as
+// large as leaves every CTA several, up to kBatchSpanGrab.
+constexpr uint64_t kBatchSpanGrab = 16;
 
-        const unsigned char *cells0 = tile + (reinterpret_cast<uintptr_t>(x.src) & 15);
-        const uint32_t cells = x.cells, runs = x.runs;
-        if (d.fixed) {
-            if (st.lane * V + V <= cells) {
-                char *o = x.dst + st.lane * WU;
-#pragma unroll 4
-                for (uint32_t run = st.group; run < runs; run += st.groups)
-                    stg<WU>(o + run_out[run], span_word<E, V>(cells0 + run_sm[run], fixed));
-            }
-        } else {
-            for (uint32_t run = st.group; run < runs; run += st.groups) {
-                char *o = x.dst + run_out[run];
-                const unsigned char *s = cells0 + run_sm[run];
-                const uint32_t head = V > 1 ? (uint32_t(reinterpret_cast<uintptr_t>(o)) & 3) / E : 0;
-#pragma unroll 4
-                for (uint32_t w = st.lane; w * V < cells + head; w += d.store_lanes) {
-                    const int32_t p = int32_t(w * V) - int32_t(head);
-                    if (p >= 0 && uint32_t(p) + V <= cells) {
-                        uint32_t f[V];
-                        span_offsets<V, LUT>(lut, p, ch0, f);
-                        stg<WU>(o + p * E, span_word<E, V>(s, f));
-                    }
-                }
-            }
-        }
-        if constexpr (V > 1) {
-            // words a span shares with its neighbours at either end: its cells, one a thread
-            if (!d.fixed || cells % V != 0) {
-                for (uint32_t i = threadIdx.x; i < runs * 2 * (V - 1); i += kThreads) {
-                    const uint32_t run = i / (2 * (V - 1)), r = i - run * 2 * (V - 1), k = r >> 1;
-                    char *o = x.dst + run_out[run];
-                    const uint32_t head = (uint32_t(reinterpret_cast<uintptr_t>(o)) & 3) / E;
-                    const uint32_t n = (r & 1) ? (cells + head) % V : (V - head) % V;  // cells of the end's word
-                    const uint32_t p = (r & 1) ? cells - 1 - k : k;
-                    if (k < n && p < cells)
-                        stg<E>(o + p * E, lds<E>(cells0 + run_sm[run] + (LUT ? uint32_t(lut[p]) : p * ch0)));
-                }
-            }
-        }
+template <int E, bool LUT>
+__device__ __noinline__ void span_range(const SpanDesc &d, uint32_t u0, uint32_t u1, unsigned char *smem, SpanUnit &unit)
+{
+    span_units<E, LUT>(d, u0, u1, 1, smem, unit, [] {});
+}
+
+__global__ void __launch_bounds__(kThreads, kSpanCtas) k_batch_span(const SpanDesc *__restrict__ spans,
+                                                                   const uint64_t *__restrict__ prefix, int n,
+                                                                   unsigned long long *counter, uint32_t grab)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ SpanUnit unit;
+    __shared__ SpanDesc d;
+    __shared__ unsigned long long s_start;
+    const uint64_t total = prefix[n];
+    for (;;) {
+        if (threadIdx.x == 0) s_start = atomicAdd(counter, (unsigned long long)grab);
         __syncthreads();
+        const uint64_t start = s_start, end = min(total, start + grab);
+        if (start >= total) break;
+        int lo = 0, hi = n - 1;  // last descriptor with prefix[lo] <= start
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (prefix[mid] <= start) lo = mid;
+            else hi = mid - 1;
+        }
+        for (uint64_t t = start; t < end; ++lo) {
+            const uint64_t base = prefix[lo], seg_end = min(end, prefix[lo + 1]);
+            for (uint32_t w = threadIdx.x; w < sizeof(SpanDesc) / 4; w += kThreads)
+                reinterpret_cast<uint32_t *>(&d)[w] = reinterpret_cast<const uint32_t *>(spans + lo)[w];
+            __syncthreads();
+            const uint32_t u0 = uint32_t(t - base), u1 = uint32_t(seg_end - base);
+            switch (d.E << 1 | d.lut) {
+                case 1 << 1 | 0: span_range<1, false>(d, u0, u1, smem, unit); break;
+                case 1 << 1 | 1: span_range<1, true>(d, u0, u1, smem, unit); break;
+                case 2 << 1 | 0: span_range<2, false>(d, u0, u1, smem, unit); break;
+                case 2 << 1 | 1: span_range<2, true>(d, u0, u1, smem, unit); break;
+                case 4 << 1 | 0: span_range<4, false>(d, u0, u1, smem, unit); break;
+                case 4 << 1 | 1: span_range<4, true>(d, u0, u1, smem, unit); break;
+                case 8 << 1 | 0: span_range<8, false>(d, u0, u1, smem, unit); break;
+                case 8 << 1 | 1: span_range<8, true>(d, u0, u1, smem, unit); break;
+                default: break;
+            }
+            t = seg_end;
+        }
     }
 }
 
@@ -261,7 +105,7 @@ cudaError_t launch_span_as(const SpanDesc &d, cudaStream_t s)
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!sms_of[dev]) {
-            e = cudaFuncSetAttribute(k_span<E, LUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+            e = cudaFuncSetAttribute(k_span<E, LUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmemMax);
             if (e != cudaSuccess) return e;
             e = cudaDeviceGetAttribute(&sms_of[dev], cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return e;
@@ -286,6 +130,23 @@ cudaError_t launch_span_as(const SpanDesc &d, cudaStream_t s)
 }
 
 }  // namespace
+
+cudaError_t launch_batch_spans(const SpanDesc *spans, const uint64_t *prefix, int n, uint64_t units, uint32_t smem,
+                               unsigned long long *counter, cudaStream_t s)
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_batch_span, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmemMax);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_span, kThreads, smem);
+    if (e != cudaSuccess) return e;
+    const uint64_t resident = uint64_t(sms) * uint64_t(std::max(per_sm, 1));
+    const uint32_t grab = uint32_t(std::max<uint64_t>(1, std::min(kBatchSpanGrab, units / (4 * resident))));
+    const uint64_t grid = std::min<uint64_t>((units + grab - 1) / grab, resident);
+    k_batch_span<<<unsigned(std::max<uint64_t>(grid, 1)), kThreads, smem, s>>>(spans, prefix, n, counter, grab);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_span(const SpanDesc &d, cudaStream_t s)
 {

@@ -26,6 +26,12 @@ inline cudaError_t launch_permute(const PermPlan &pl, cudaStream_t s)
     return pl.use_span ? launch_span(pl.span, s) : launch_single(pl.op, nullptr, s);
 }
 
+// The span copies of a batch (device arrays of n descriptors and of the prefix
+// sums of their units; smem: the largest descriptor's shared memory; counter
+// zeroed before).
+cudaError_t launch_batch_spans(const SpanDesc *spans, const uint64_t *prefix, int n, uint64_t units, uint32_t smem,
+                               unsigned long long *counter, cudaStream_t s);
+
 // The L2-resident bucketed reorder (k_reorder_l2.cu) of a gather op with l2 set.
 cudaError_t launch_reorder_l2(const OpDesc &op, cudaStream_t s);
 

@@ -358,7 +358,7 @@ static bool plan_box(const std::vector<Axis> &ax, int64_t E, uintptr_t da, uintp
 // given in order (slowest first) with their input byte strides; src already
 // points at the element of output index 0.  The output is contiguous.
 static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, const std::vector<Axis> &in_axes,
-                              uint64_t total, PermPlan &pl, std::string &err)
+                              uint64_t total, PermPlan &pl, std::string &err, bool in_batch)
 {
     rearr_permute_info &info = pl.info;
     const uint64_t bytes = total * elem_bytes;
@@ -695,6 +695,11 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     if (W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
     const bool sparse = op.cls == OC_TILE && 3 * n_cells < 2 * op.units * uint64_t(t.TA) * t.TB;
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
+    if (in_batch) {
+        pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || sparse || (op.cls == OC_TILE && narrow)) &&
+                            plan_span(ax, cell, static_cast<char *>(dst), src, pl.batch_span, false);
+        return REARR_OK;
+    }
     pl.use_planes = (thin || narrow || sparse) &&
                     plan_planes(ax, cell, static_cast<char *>(dst), src, pl.planes_op, pl.planes);
     if (!pl.use_planes && ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16))))
@@ -765,7 +770,7 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
 }
 
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank, const int64_t *dims,
-                          const int *perm, PermPlan &pl, std::string &err)
+                          const int *perm, PermPlan &pl, std::string &err, bool in_batch)
 {
     std::memset(&pl, 0, sizeof(pl));
     rearr_permute_info &info = pl.info;
@@ -807,12 +812,12 @@ rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int ran
     for (int i = rank - 2; i >= 0; --i) s[i] = s[i + 1] * dims[i + 1];
     std::vector<Axis> ax;
     for (int i = 0; i < rank; ++i) ax.push_back(Axis{dims[perm[i]], s[perm[i]]});
-    return plan_axes(dst, static_cast<const char *>(src), elem_bytes, ax, total, pl, err);
+    return plan_axes(dst, static_cast<const char *>(src), elem_bytes, ax, total, pl, err, in_batch);
 }
 
 rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int rank_in, const int64_t *dims,
                              int rank_out, const int *order, const int64_t *base, const int64_t *range,
-                             PermPlan &pl, std::string &err)
+                             PermPlan &pl, std::string &err, bool in_batch)
 {
     std::memset(&pl, 0, sizeof(pl));
     pl.info.plane_a = -1;
@@ -862,7 +867,7 @@ rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int 
     for (int a = 0; a < rank_in; ++a) off += base[a] * s[a];
     std::vector<Axis> ax;
     for (int i = 0; i < rank_out; ++i) ax.push_back(Axis{range[order[i]], s[order[i]]});
-    return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err);
+    return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err, in_batch);
 }
 
 rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_t n, size_t elem_bytes,

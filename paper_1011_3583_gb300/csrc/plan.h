@@ -27,6 +27,8 @@ struct PermPlan {
     OpDesc planes_op;
     char *planes[kInlineK];
     SpanDesc span;
+    SpanDesc batch_span;      // the span copy a captured batch runs instead of op,
+    bool use_batch_span;      // if it was asked for and there is one
 };
 
 struct InterlacePlan {
@@ -36,11 +38,13 @@ struct InterlacePlan {
 
 // Each returns REARR_OK or REARR_EINVAL (with a message in err).  A plan with
 // op.units == 0 is a no-op.
+// batch: plan for a captured batch (batch_span) instead of a single call.
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank,
-                          const int64_t *dims, const int *perm, PermPlan &pl, std::string &err);
+                          const int64_t *dims, const int *perm, PermPlan &pl, std::string &err,
+                          bool batch = false);
 rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int rank_in, const int64_t *dims,
                              int rank_out, const int *order, const int64_t *base, const int64_t *range,
-                             PermPlan &pl, std::string &err);
+                             PermPlan &pl, std::string &err, bool batch = false);
 // Gather dst[i] = src[idx[i]] (or, with scatter, dst[idx[i]] = src[i]) with
 // idx_bytes-byte (4 or 8) indices.
 rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_t n,
@@ -55,8 +59,9 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
                  char *(&planes)[kInlineK]);
 
 // Span copy of the canonical axes (output order, slowest first; input strides
-// in bytes; one E-byte word a cell): false where it does not apply.
-bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d);
+// in bytes; one E-byte word a cell): false where it does not apply.  alone: the
+// op has the GPU to itself, so a small one is cut into units that fill it.
+bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone = true);
 
 // A fast tile planned with the 32 KB payload re-planned with the 16 KB tile of
 // the same row length (the batched kernel holds two 16 KB tiles per CTA).

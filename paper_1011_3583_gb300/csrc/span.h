@@ -25,6 +25,7 @@ namespace rearr {
 constexpr int kSpanAxes = 4;        // axes of either chain
 constexpr int kSpanOuter = 8;       // unit-index digits
 constexpr int kSpanMaxSpans = 512;  // input / output spans per unit
+constexpr int kSpanSmemMax = 96 * 1024;  // shared memory of a unit, at most (60 KB of spans, then the tables)
 constexpr int kSpanMaxLut = 8192;   // cells of an output span that runs over several axes
 
 struct SpanDesc {

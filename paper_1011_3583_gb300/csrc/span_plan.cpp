@@ -23,7 +23,7 @@ struct Chain {
 
 }  // namespace
 
-bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d)
+bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone)
 {
     const int R = int(ax.size());
     if (R > kMaxRank || R < 2) return false;
@@ -35,7 +35,7 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
         K[i] = 0;
         total *= uint64_t(ax[i].extent);
     }
-    const uint64_t box = std::max(kSpanMinBoxBytes, std::min(kSpanBoxBytes, total / kSpanFillUnits));
+    const uint64_t box = alone ? std::max(kSpanMinBoxBytes, std::min(kSpanBoxBytes, total / kSpanFillUnits)) : kSpanBoxBytes;
     const int64_t vmax = int64_t(box) / E;  // cells of a unit
     int64_t target = E;                     // bytes wanted of each span: an even split of the unit
     while (target * target < vmax * E * E) target *= 2;

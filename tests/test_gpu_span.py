@@ -109,3 +109,54 @@ def test_capture(lr, orc):
         sync()
         for a, (e, dims, perm), (_, d) in zip(srcs, cases, bufs):
             assert np.array_equal(d.download(), orc.permute(a, e, dims, perm)), (seed, e, dims, perm)
+
+
+def test_large_batch(lr, orc):
+    """A plan large enough to be split over the batch's kernels: every op as its
+    single call would compute it, replayed on new contents."""
+    plan = lr.Plan()
+    ops = []
+    for i in range(20):  # 2048 units each
+        e, n = (1, 2, 1, 4)[i % 4], (1 << 22) - i
+        ops.append(dict(kind="scatter" if i % 5 == 4 else "reorder", e=e, n=n, idx=synth.random_permutation(i, n)))
+    for i in range(60):
+        dims, perm = SPANS[i % len(SPANS)]
+        ops.append(dict(kind="permute", e=(1, 2, 4, 8)[i % 4], n=int(np.prod(dims)), dims=dims, perm=perm))
+    for dims, perm in (([64, 64, 128], [2, 1, 0]), ([128, 40, 256], [1, 0, 2]), ([70000], [0])):
+        ops.append(dict(kind="permute", e=4, n=int(np.prod(dims)), dims=dims, perm=perm))
+    for k in (2, 3, 9):
+        ops.append(dict(kind="interlace", e=2, n=20000 + k, k=k))
+    for op in ops:
+        e, n = op["e"], op["n"]
+        op["in"] = [DevBuf(n * e) for _ in range(op.get("k", 1))]
+        op["out"] = DevBuf(n * e * op.get("k", 1), fill=0x55)
+        if op["kind"] in ("reorder", "scatter"):
+            op["didx"] = to_dev(op["idx"])
+            add = plan.add_reorder if op["kind"] == "reorder" else plan.add_scatter
+            add(op["out"].ptr, op["in"][0].ptr, op["didx"].ptr, n, e)
+        elif op["kind"] == "permute":
+            plan.add_permute(op["out"].ptr, op["in"][0].ptr, e, op["dims"], op["perm"])
+        else:
+            plan.add_interlace(op["out"].ptr, [b.ptr for b in op["in"]], n, e)
+    assert plan.stats()[1] > 40000
+    plan.finalize()
+    for replay in range(2):
+        for i, op in enumerate(ops):
+            op["src"] = [synth.random_elements(1000 * replay + i + 7 * j, op["n"], op["e"]) for j in range(len(op["in"]))]
+            for b, a in zip(op["in"], op["src"]):
+                b.upload(a)
+        plan.run()
+        sync()
+        for op in ops:
+            e, n, src = op["e"], op["n"], op["src"]
+            if op["kind"] == "reorder":
+                want = orc.reorder(src[0], op["idx"], e)
+            elif op["kind"] == "scatter":
+                inv = np.empty(n, dtype=np.uint32)
+                inv[op["idx"]] = np.arange(n, dtype=np.uint32)
+                want = orc.reorder(src[0], inv, e)
+            elif op["kind"] == "permute":
+                want = orc.permute(src[0], e, op["dims"], op["perm"])
+            else:
+                want = orc.interlace(src, n, e)
+            assert np.array_equal(op["out"].download(), want), (replay, op["kind"], e, n, op.get("dims"))
