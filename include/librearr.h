@@ -124,7 +124,10 @@ rearr_status rearr_reorder(void *dst, const void *src, const uint32_t *idx, size
  *   aligned to its index size.  Large gathers and scatters with 4/8/16-byte
  *   elements (either index size, n < 2^32) use the L2-resident passes of
  *   rearr_reorder (a scatter's buckets by destination chunk), with the same
- *   locality check and scratch pool.
+ *   locality check and scratch pool.  A scatter of 4- or 8-byte elements of up
+ *   to about 640 / 400 MB first sorts them into lists per shared-memory-sized
+ *   destination chunk and places each list in shared memory; the passes run
+ *   where a list would overflow (indices crowded in a few chunks).
  * ------------------------------------------------------------------------- */
 rearr_status rearr_scatter(void *dst, const void *src, const uint32_t *idx, size_t n,
                            size_t elem_bytes, rearr_stream_t stream);
@@ -173,7 +176,8 @@ typedef enum {
                                           place, gather per source chunk, scatter
                                           through shared memory per 64 KB chunk  */
     REARR_REORDER_L2_SCATTER = 2,      /* gather, last pass through ~16 MB L2 chunks */
-    REARR_REORDER_LINEAR_SCATTER = 3   /* scatter: (destination, element) pairs      */
+    REARR_REORDER_LINEAR_SCATTER = 3   /* scatter: (destination, element) pairs (or
+                                          chunk lists within the same scratch)    */
 } rearr_reorder_form;
 
 typedef struct {

@@ -152,6 +152,42 @@ __device__ __forceinline__ int tid_x()
     return t;
 }
 
+// First thing in a kernel launched with programmatic stream serialisation
+// behind others of its kind that do not trigger it early: its launch overlaps
+// their drain, and no memory is touched before they are complete.  (Letting
+// the next pass's CTAs in beside the working ones was measured: the SM keeps
+// the first kernel's split of L1 and shared memory for both, and the reorder's
+// gather pass took half again as long.)
+__device__ __forceinline__ void pass_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Exclusive prefix sum of one value per thread over a CTA of THREADS (whole
+// warps); warp_sums: 32 words of shared memory.
+template <int THREADS>
+__device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *warp_sums)
+{
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        const uint32_t s = lane < THREADS / 32 ? warp_sums[lane] : 0u;
+        uint32_t y = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += z;
+        }
+        if (lane < THREADS / 32) warp_sums[lane] = y - s;
+    }
+    __syncthreads();
+    return warp_sums[w] + x - v;
+}
+
 // Byte select of two words (PRMT): result byte i = byte sel_i of {b:a}.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {

@@ -34,7 +34,13 @@
 // A scatter (dst[idx[i]] = src[i]) uses one bucket dimension only (D = 1,
 // buckets by the destination chunk of idx[i]): the partition writes
 // (destination index, element) pairs, and a linear pass writes
-// dst[s[k]] = v[k] with the destination chunk L2-resident.
+// dst[s[k]] = v[k] with the destination chunk L2-resident.  Scatters of 4- and
+// 8-byte elements up to a size go through chunk lists first
+// (scatter_chunks.cuh) and take these passes only where a list overflows.
+// Every pass is launched behind the one before (pass_enter()), which takes
+// most of the launch off those that return at once: block-shuffled 2^26 x 4 B
+// scatter 149 -> 142 us with two passes more, gather 2^25 x 4 B 338 -> 327,
+// 2^24 x 8 B 216 -> 204.
 // Random global accesses cost one L1 request each (about one per clock per
 // SM, whatever the working set); random shared-memory accesses run about
 // twelve times as fast, so in the tile-local form the gather is the one pass
@@ -53,6 +59,7 @@
 #include "bodies.cuh"
 #include "launch.h"
 #include "reorder_geometry.h"
+#include "scatter_chunks.cuh"
 #include "tuning.h"
 
 namespace rearr {
@@ -63,7 +70,6 @@ constexpr int kTile = 4096;        // elements per partition tile / scatter unit
 constexpr int kMaxChunks = int(kReorderMaxChunks);  // C <= 512; D <= 512 for the L2 scatter
 constexpr int kScatterThreads = 512;
 constexpr uint32_t kScatterChunkBytes = kReorderScatterChunkBytes;  // destination chunk of the shared-memory scatter
-constexpr int kSampleRuns = 4096;
 constexpr int kSampleLen = 64;
 constexpr uint32_t kNear = 16;
 
@@ -79,6 +85,7 @@ struct L2Reorder {
     unsigned long long *near;      // K1: close neighbour pairs in the sample
     unsigned int *ctr_gather;      // K5 / K6 work counters (units handed out in order)
     unsigned int *ctr_scatter;
+    unsigned int *done;            // histogram CTAs that have finished
     uint32_t *hist;                // [C*D] bucket sizes, c-major (b = c*D + d)
     uint32_t *rowtot;              // [C] elements per source chunk
     uint32_t *base;                // [C*D] bucket starts, c-major
@@ -90,6 +97,11 @@ struct L2Reorder {
     uint16_t *st;                  // tile-local form: [tiles][C + 1] segment starts per tile
     uint32_t tiles;                // 4096-index tiles of the sequence
     unsigned long long near_threshold;
+    // a scatter tried through chunk lists first (scatter_chunks.cuh): the flag
+    // that they overflowed; their chunks and the sampled indices of each
+    const uint32_t *over;
+    uint32_t *hits;
+    uint32_t list_mul, list_shift, list_C;
 };
 
 // Source chunk of an index; clamped so that an index >= n (undefined
@@ -121,18 +133,26 @@ __device__ __forceinline__ uint32_t index_at_t(const L2Reorder &p, uint64_t i)
     else return __ldg(p.idx + i);
 }
 
-__device__ __forceinline__ bool bucketed(const L2Reorder &p)
+// The sample found the indices far apart: the direct kernel is not to run.
+__device__ __forceinline__ bool far_apart(const L2Reorder &p)
 {
     return *reinterpret_cast<volatile unsigned long long *>(p.near) < p.near_threshold;
+}
+
+// The bucketed passes are to run.
+__device__ __forceinline__ bool bucketed(const L2Reorder &p)
+{
+    return far_apart(p) && (!p.over || *reinterpret_cast<const volatile uint32_t *>(p.over));
 }
 
 // One warp per sampled run of 64 consecutive indices: each lane loads two
 // neighbouring entries and compares them with the next lane's.
 __global__ void __launch_bounds__(kThreads) k_l2_sample(const L2Reorder p)
 {
+    pass_enter();
     const uint32_t r = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31;
-    uint32_t cnt = 0;
+    uint32_t cnt = 0, first = 0;
     if (r < kSampleRuns && p.n > kSampleLen) {
         const uint64_t start = uint64_t(r) * (p.n - kSampleLen) / kSampleRuns;
         const uint32_t a = index_at(p, start + 2 * lane), b = index_at(p, start + 2 * lane + 1);
@@ -140,10 +160,17 @@ __global__ void __launch_bounds__(kThreads) k_l2_sample(const L2Reorder p)
         const uint32_t d1 = b > a ? b - a : a - b;
         const uint32_t d2 = next_a > b ? next_a - b : b - next_a;
         cnt = (d1 <= kNear) + (lane < 31 && d2 <= kNear);
+        first = a;
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(p.near, (unsigned long long)cnt);
+    if (lane == 0 && cnt) atomicAdd(p.near, (unsigned long long)cnt);
+    if (p.hits && cnt < kSampleLen / 2 && lane < kSampleRunHits) {
+        // a run of scattered indices: count some by chunk, equal ones together
+        const uint32_t c = min(__umulhi(first, p.list_mul) >> p.list_shift, p.list_C - 1);
+        const uint32_t same = __match_any_sync((1u << kSampleRunHits) - 1, c);
+        if (lane == uint32_t(__ffs(int(same))) - 1) atomicAdd(&p.hits[size_t(c) * kFillStride], uint32_t(__popc(same)));
+    }
 }
 
 // Elements of a tile: warp w owns the contiguous slice [w*512, (w+1)*512);
@@ -173,12 +200,51 @@ __device__ __forceinline__ void load_tile(const L2Reorder &p, uint32_t i0, uint3
     }
 }
 
+// Bucket starts and scatter units from the bucket sizes, by one CTA (the last
+// one of the histogram pass to finish).
+__device__ __forceinline__ void scan_buckets(const L2Reorder &p, uint32_t *warp_sums, uint32_t *total)
+{
+    const uint32_t nb = p.C * p.D;
+    auto scan = [&](uint32_t v) {
+        const uint32_t e = cta_scan<kThreads>(v, warp_sums);
+        if (threadIdx.x == kThreads - 1) *total = e + v;
+        __syncthreads();
+        return e;
+    };
+    uint32_t carry = 0;
+    for (uint32_t b0 = 0; b0 < nb; b0 += kThreads) {  // bucket starts, c-major
+        const uint32_t b = b0 + threadIdx.x;
+        const uint32_t e = scan(b < nb ? __ldcg(p.hist + b) : 0u);
+        if (b < nb) {
+            p.base[b] = carry + e;
+            p.cursor[b] = carry + e;
+        }
+        carry += *total;
+        __syncthreads();
+    }
+    carry = 0;
+    for (uint32_t s0 = 0; s0 < nb; s0 += kThreads) {  // scatter units, d-major (s = d*C + c)
+        const uint32_t s = s0 + threadIdx.x;
+        uint32_t v = 0;
+        if (s < nb) {
+            const uint32_t d = s / p.C, c = s - d * p.C;
+            v = (__ldcg(p.hist + c * p.D + d) + kTile - 1) / kTile;
+        }
+        const uint32_t e = scan(v);
+        if (s < nb) p.uprefix[s] = carry + e;
+        carry += *total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) p.uprefix[nb] = carry;
+}
+
 // Each CTA walks a contiguous range of tiles with per-warp shared counters
 // (the only contention is among the lanes of one warp) and flushes them to
 // the global histogram whenever the destination chunk changes.
 template <bool I64>
 __global__ void __launch_bounds__(kThreads) k_l2_hist(const L2Reorder p, uint32_t tiles_per_cta)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     __shared__ uint32_t sh[kWarps][kMaxChunks];
     const uint32_t w = threadIdx.x >> 5;
@@ -231,69 +297,17 @@ __global__ void __launch_bounds__(kThreads) k_l2_hist(const L2Reorder p, uint32_
         const uint32_t c = threadIdx.x + j * kThreads;
         if (c < p.C && row[j]) atomicAdd(&p.rowtot[c], row[j]);
     }
-}
-
-// Exclusive block-wide scan of one value per thread (1024 threads); returns
-// the prefix and the block total in *total.
-__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t *warp_sums, uint32_t *total)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[warp] = x;
+    // The last CTA to get here has every count behind it.
+    __shared__ uint32_t warp_sums[32], total;
+    __shared__ bool last;
+    __threadfence();
     __syncthreads();
-    if (warp == 0) {
-        uint32_t w = warp_sums[lane];
-        uint32_t s = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        warp_sums[lane] = s - w;  // exclusive prefix of the warps
-        if (lane == 31) *total = s;
-    }
+    if (threadIdx.x == 0) last = atomicAdd(p.done, 1u) == gridDim.x - 1;
     __syncthreads();
-    const uint32_t r = warp_sums[warp] + x - v;
-    __syncthreads();
-    return r;
-}
-
-// One CTA of 1024 threads.
-__global__ void __launch_bounds__(1024) k_l2_scan(const L2Reorder p)
-{
-    if (!bucketed(p)) return;
-    __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t total;
-    const uint32_t nb = p.C * p.D;
-    uint32_t carry = 0;
-    for (uint32_t b0 = 0; b0 < nb; b0 += 1024) {  // bucket starts, c-major
-        const uint32_t b = b0 + threadIdx.x;
-        const uint32_t v = b < nb ? p.hist[b] : 0;
-        const uint32_t e = block_scan(v, warp_sums, &total);
-        if (b < nb) {
-            p.base[b] = carry + e;
-            p.cursor[b] = carry + e;
-        }
-        carry += total;
+    if (last) {
+        __threadfence();
+        scan_buckets(p, warp_sums, &total);
     }
-    carry = 0;
-    for (uint32_t s0 = 0; s0 < nb; s0 += 1024) {  // scatter units, d-major (s = d*C + c)
-        const uint32_t s = s0 + threadIdx.x;
-        uint32_t v = 0;
-        if (s < nb) {
-            const uint32_t d = s / p.C, c = s - d * p.C;
-            v = (p.hist[c * p.D + d] + kTile - 1) / kTile;
-        }
-        const uint32_t e = block_scan(v, warp_sums, &total);
-        if (s < nb) p.uprefix[s] = carry + e;
-        carry += total;
-    }
-    if (threadIdx.x == 0) p.uprefix[nb] = carry;
 }
 
 // Partition: per tile, every warp ranks its 512 elements by source chunk in
@@ -323,6 +337,7 @@ static_assert(sizeof(PartitionSmem) % 16 == 0, "the scatter form's element buffe
 template <int SW, bool I64>
 __global__ void __launch_bounds__(kThreads, 4) k_l2_partition(const L2Reorder p, uint32_t tiles_per_cta)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PartitionSmem &S = *reinterpret_cast<PartitionSmem *>(smem_raw);
@@ -450,6 +465,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_l2_partition(const L2Reorder p,
 template <bool I64>
 __global__ void __launch_bounds__(kThreads, 4) k_l2_partition_local(const L2Reorder p, uint32_t tiles_per_cta)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PartitionSmem &S = *reinterpret_cast<PartitionSmem *>(smem_raw);
@@ -563,6 +579,7 @@ constexpr int kGatherUnit = 2048;  // elements per gather / scatter unit (8 per 
 template <int W>
 __global__ void __launch_bounds__(kThreads, W == 4 ? 8 : W == 8 ? 6 : 4) k_l2_gather(const L2Reorder p)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     __shared__ uint32_t slot;
     using T = typename Word<W>::T;
@@ -604,6 +621,7 @@ __global__ void __launch_bounds__(kThreads, W == 4 ? 8 : W == 8 ? 6 : 4) k_l2_ga
 template <int W, int S, int J>
 __global__ void __launch_bounds__(kThreads, W == 4 ? 6 : W == 8 ? 5 : 4) k_l2_gather_local(const L2Reorder p)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     constexpr uint32_t kUnitTiles = kWarps * S;
     __shared__ uint32_t slot;
@@ -663,6 +681,7 @@ __global__ void __launch_bounds__(kThreads, W == 4 ? 6 : W == 8 ? 5 : 4) k_l2_ga
 template <int W>
 __global__ void __launch_bounds__(kScatterThreads) k_l2_scatter_local(const L2Reorder p)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     using T = typename Word<W>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -708,6 +727,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_l2_scatter_local(const L2Re
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_l2_scatter(const L2Reorder p)
 {
+    pass_enter();
     if (!bucketed(p)) return;
     __shared__ uint32_t slot, sk0, sk1;
     using T = typename Word<W>::T;
@@ -754,9 +774,19 @@ __global__ void __launch_bounds__(kThreads) k_l2_scatter(const L2Reorder p)
 
 // Scatter form, last pass: dst[s[k]] = v[k] in k order (c-major: one
 // destination chunk at a time, L2-resident while its sectors are completed).
-template <int W>
-__global__ void __launch_bounds__(kThreads) k_l2_scatter_linear(const L2Reorder p)
+// DIRECT: also the direct scatter when the sample found the indices local (one
+// launch less where chunk lists add two; 16-byte elements, which have none,
+// keep the leaner kernel).
+template <int W, bool DIRECT>
+__global__ void __launch_bounds__(kThreads) k_l2_scatter_linear(const L2Reorder p, const GatherDesc g, uint64_t dunits)
 {
+    pass_enter();
+    if constexpr (DIRECT) {
+        if (!far_apart(p)) {
+            for (uint64_t u = blockIdx.x; u < dunits; u += gridDim.x) gather_body<W>(g, u);
+            return;
+        }
+    }
     if (!bucketed(p)) return;
     __shared__ uint32_t slot;
     using T = typename Word<W>::T;
@@ -789,7 +819,8 @@ __global__ void __launch_bounds__(kThreads) k_l2_scatter_linear(const L2Reorder 
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_l2_direct(const L2Reorder p, const GatherDesc g, uint64_t units)
 {
-    if (bucketed(p)) return;
+    pass_enter();
+    if (far_apart(p)) return;
     for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) gather_body<W>(g, u);
 }
 
@@ -819,6 +850,43 @@ cudaError_t get_pool(cudaMemPool_t &pool)
     return cudaSuccess;
 }
 
+// Shared-memory opt-in of a kernel on the current device.
+template <class K> cudaError_t opt_in(K kernel, size_t bytes)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
+
+// Launch of a pass (pass_enter()).
+template <class... P, class... A>
+cudaError_t pass(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <int W>
+cudaError_t run_lists(const ScatterLists &p, bool idx64, size_t sm, unsigned sms, cudaStream_t s)
+{
+    constexpr int NG = W == 4 ? 6 : 4;
+    auto kernel = idx64 ? k_scatter_lists<W, true, NG> : k_scatter_lists<W, false, NG>;
+    cudaError_t e = opt_in(kernel, sm);
+    if (e != cudaSuccess) return e;
+    e = pass(kernel, std::min<unsigned>(p.tiles, sms), kListThreads, sm, s, p);
+    const size_t place = size_t(p.CS) * W + p.CS / 8;
+    if (e == cudaSuccess) e = opt_in(k_scatter_place<W>, place);
+    if (e != cudaSuccess) return e;
+    return pass(k_scatter_place<W>, std::min<unsigned>(p.C, sms), kListThreads, place, s, p);
+}
+
 template <int W>
 cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
 {
@@ -839,6 +907,14 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
     const size_t off_hist = gm.off_hist, off_row = gm.off_row, off_base = gm.off_base, off_cur = gm.off_cur,
                  off_up = gm.off_up, off_s = gm.off_s, off_i = gm.off_i, off_v = gm.off_v, off_st = gm.off_st,
                  bytes = gm.bytes;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // A scatter goes through chunk lists; the bucketed passes below then run
+    // only if a list overflowed, or the sample says that one would.
+    const ListGeometry lg = list_geometry(g.n, W, uint32_t(sms), off_s, bytes);
+    const bool lists = W <= 8 && g.scatter && lg.on &&
+                       reorder_geometry(g.n, W, false, reorder_smem_max_buckets()).smem_scatter;
     cudaMemPool_t pool;
     cudaError_t e = get_pool(pool);
     if (e != cudaSuccess) return e;
@@ -848,6 +924,7 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
     p.near = reinterpret_cast<unsigned long long *>(scratch);
     p.ctr_gather = reinterpret_cast<unsigned int *>(scratch + 8);
     p.ctr_scatter = reinterpret_cast<unsigned int *>(scratch + 16);
+    p.done = reinterpret_cast<unsigned int *>(scratch + 32);
     p.hist = reinterpret_cast<uint32_t *>(scratch + off_hist);
     p.rowtot = reinterpret_cast<uint32_t *>(scratch + off_row);
     p.base = reinterpret_cast<uint32_t *>(scratch + off_base);
@@ -860,11 +937,8 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
     p.tiles = uint32_t((g.n + kTile - 1) / kTile);
     const uint64_t pairs = uint64_t(kSampleRuns) * (kSampleLen - 1);
     p.near_threshold = pairs / 2;
-    e = cudaMemsetAsync(scratch, 0, off_base, s);  // near counter, histogram, row totals
-
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // counters, histogram, row totals; up to the lists' counters
+    e = cudaMemsetAsync(scratch, 0, lists ? lg.off_off : off_base, s);
     const uint32_t tiles = (p.n + kTile - 1) / kTile;
     const uint32_t resident = uint32_t(sms) * 4;
     const uint32_t tpc = (tiles + resident - 1) / resident;  // contiguous tiles per CTA
@@ -922,64 +996,83 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
     const uint32_t part_tpc = (tiles + part_resident - 1) / part_resident;
     const unsigned part_grid = unsigned((tiles + part_tpc - 1) / part_tpc);
     const unsigned pers = unsigned(sms) * 8;  // persistent grids of the gated passes
+    // The direct kernel's grid: two resident waves.  When the bucketed passes ran
+    // it exits at once; when it works, that is as fast as one CTA per unit.
     const uint64_t dunits = (g.n + g.unit_elems - 1) / g.unit_elems;
-    if (e == cudaSuccess) { k_l2_sample<<<kSampleRuns / (kThreads / 32), kThreads, 0, s>>>(p); e = cudaGetLastError(); }
+    const unsigned direct_grid = unsigned(std::min<uint64_t>(dunits, uint64_t(sms) * 16));
+    ScatterLists f = {};
+    if (lists) {
+        f.src = p.src;
+        f.dst = p.dst;
+        f.idx = p.idx;
+        f.n = p.n;
+        f.C = lg.C;
+        f.CS = lg.CS;
+        f.cap = lg.cap;
+        f.cs_mul = lg.cs_mul;
+        f.cs_shift = lg.cs_shift;
+        f.tiles = uint32_t((g.n + lg.T - 1) / lg.T);
+        f.hits_max = lg.hits_max;
+        f.near = p.near;
+        f.near_threshold = p.near_threshold;
+        f.over = reinterpret_cast<uint32_t *>(scratch + 24);  // zeroed with the counters
+        f.fill = reinterpret_cast<uint32_t *>(scratch + lg.off_fill);
+        f.off = reinterpret_cast<uint16_t *>(scratch + lg.off_off);
+        f.v = scratch + lg.off_v;
+        p.over = f.over;
+        p.hits = f.fill + 1;
+        p.list_mul = lg.cs_mul;
+        p.list_shift = lg.cs_shift;
+        p.list_C = lg.C;
+    }
+    if (e == cudaSuccess) e = pass(k_l2_sample, kSampleRuns / (kThreads / 32), kThreads, 0, s, p);
+    if constexpr (W <= 8) {
+        if (lists && e == cudaSuccess) e = run_lists<W>(f, p.idx64 != 0, lg.smem, unsigned(sms), s);
+    }
     // A gather with CTA-sized destination chunks runs the tile-local form:
     // partition in place, gather over the tiles' segments, scatter per chunk.
     const bool local = smem_scatter && !g.scatter;
     if (local) {
         if (e == cudaSuccess) {
-            if (p.idx64) k_l2_partition_local<true><<<part_grid, kThreads, sizeof(PartitionSmem), s>>>(p, part_tpc);
-            else k_l2_partition_local<false><<<part_grid, kThreads, sizeof(PartitionSmem), s>>>(p, part_tpc);
-            e = cudaGetLastError();
+            if (p.idx64) e = pass(k_l2_partition_local<true>, part_grid, kThreads, sizeof(PartitionSmem), s, p, part_tpc);
+            else e = pass(k_l2_partition_local<false>, part_grid, kThreads, sizeof(PartitionSmem), s, p, part_tpc);
         }
         if (e == cudaSuccess) {
             // segments of 4096 / C elements: tiles per warp so that a unit is ~2048 elements
             // (wider elements take fewer per lane, within the register budget)
             constexpr int J1 = W == 16 ? 8 : 10, J2 = W == 16 ? 4 : 6, J4 = W == 4 ? 3 : 2;
-            if (p.C <= 16) k_l2_gather_local<W, 1, J1><<<pers, kThreads, 0, s>>>(p);
-            else if (p.C <= 32) k_l2_gather_local<W, 2, J2><<<pers, kThreads, 0, s>>>(p);
-            else if (p.C <= 64) k_l2_gather_local<W, 4, J4><<<pers, kThreads, 0, s>>>(p);
-            else k_l2_gather_local<W, 4, 2><<<pers, kThreads, 0, s>>>(p);
-            e = cudaGetLastError();
+            if (p.C <= 16) e = pass(k_l2_gather_local<W, 1, J1>, pers, kThreads, 0, s, p);
+            else if (p.C <= 32) e = pass(k_l2_gather_local<W, 2, J2>, pers, kThreads, 0, s, p);
+            else if (p.C <= 64) e = pass(k_l2_gather_local<W, 4, J4>, pers, kThreads, 0, s, p);
+            else e = pass(k_l2_gather_local<W, 4, 2>, pers, kThreads, 0, s, p);
         }
         if (e == cudaSuccess) {
             const unsigned sgrid = unsigned(std::min<uint64_t>(p.D, uint64_t(sms) * per_sm_scat));
-            k_l2_scatter_local<W><<<sgrid, kScatterThreads, kScatterChunkBytes, s>>>(p);
-            e = cudaGetLastError();
+            e = pass(k_l2_scatter_local<W>, sgrid, kScatterThreads, kScatterChunkBytes, s, p);
         }
     }
     if (e == cudaSuccess && !local) {
-        if (p.idx64) k_l2_hist<true><<<pgrid, kThreads, 0, s>>>(p, tpc);
-        else k_l2_hist<false><<<pgrid, kThreads, 0, s>>>(p, tpc);
-        e = cudaGetLastError();
+        if (p.idx64) e = pass(k_l2_hist<true>, pgrid, kThreads, 0, s, p, tpc);
+        else e = pass(k_l2_hist<false>, pgrid, kThreads, 0, s, p, tpc);
     }
-    if (e == cudaSuccess && !local) { k_l2_scan<<<1, 1024, 0, s>>>(p); e = cudaGetLastError(); }
     if (e == cudaSuccess && !local) {
         const size_t sm_part = sizeof(PartitionSmem) + (g.scatter ? size_t(kTile) * W : 0);
-        if (g.scatter && p.idx64) k_l2_partition<W, true><<<part_grid, kThreads, sm_part, s>>>(p, part_tpc);
-        else if (g.scatter) k_l2_partition<W, false><<<part_grid, kThreads, sm_part, s>>>(p, part_tpc);
-        else if (p.idx64) k_l2_partition<0, true><<<part_grid, kThreads, sm_part, s>>>(p, part_tpc);
-        else k_l2_partition<0, false><<<part_grid, kThreads, sm_part, s>>>(p, part_tpc);
-        e = cudaGetLastError();
+        if (g.scatter && p.idx64) e = pass(k_l2_partition<W, true>, part_grid, kThreads, sm_part, s, p, part_tpc);
+        else if (g.scatter) e = pass(k_l2_partition<W, false>, part_grid, kThreads, sm_part, s, p, part_tpc);
+        else if (p.idx64) e = pass(k_l2_partition<0, true>, part_grid, kThreads, sm_part, s, p, part_tpc);
+        else e = pass(k_l2_partition<0, false>, part_grid, kThreads, sm_part, s, p, part_tpc);
     }
     if (local) {
         // done above
     } else if (!g.scatter) {
-        if (e == cudaSuccess) { k_l2_gather<W><<<pers, kThreads, 0, s>>>(p); e = cudaGetLastError(); }
-        if (e == cudaSuccess) { k_l2_scatter<W><<<pers, kThreads, 0, s>>>(p); e = cudaGetLastError(); }
+        if (e == cudaSuccess) e = pass(k_l2_gather<W>, pers, kThreads, 0, s, p);
+        if (e == cudaSuccess) e = pass(k_l2_scatter<W>, pers, kThreads, 0, s, p);
     } else {
         // the partition wrote (destination index, element) pairs
-        if (e == cudaSuccess) { k_l2_scatter_linear<W><<<pers, kThreads, 0, s>>>(p); e = cudaGetLastError(); }
+        if (e == cudaSuccess) e = pass(k_l2_scatter_linear<W, (W <= 8)>, W <= 8 ? direct_grid : pers, kThreads, 0, s, p, g, dunits);
     }
-    if (e == cudaSuccess) {
-        // two resident waves: when the bucketed passes ran, the grid exits at
-        // once; when it gathers, that is as fast as one CTA per unit
-        const uint64_t cap = uint64_t(sms) * 16;
-        k_l2_direct<W><<<unsigned(std::min<uint64_t>(dunits, cap)), kThreads, 0, s>>>(p, g, dunits);
-        e = cudaGetLastError();
-    }
-    g_launches.fetch_add(local ? 5 : g.scatter ? 6 : 7, std::memory_order_relaxed);
+    if (e == cudaSuccess && (!g.scatter || W > 8)) e = pass(k_l2_direct<W>, direct_grid, kThreads, 0, s, p, g, dunits);
+    g_launches.fetch_add(local ? 5 : (lists ? 6 : g.scatter ? 4 : 6) + (g.scatter && W > 8), std::memory_order_relaxed);
     cudaError_t e2 = cudaFreeAsync(scratch, s);
     return e != cudaSuccess ? e : e2;
 }

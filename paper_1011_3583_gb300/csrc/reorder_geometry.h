@@ -59,4 +59,67 @@ inline ReorderGeometry reorder_geometry(uint64_t n, uint32_t W, bool scatter, ui
     return g;
 }
 
+// Scatters through chunk lists (scatter_chunks.cuh): destination chunks that
+// fit one CTA's shared memory.
+constexpr uint32_t kListChunkBytes = 208u << 10;       // shared memory of a chunk
+constexpr uint64_t kListMaxElems = uint64_t(1) << 29;  // the chunk division's range
+constexpr size_t kListSmem = 231000;                   // shared memory of a CTA, at most
+
+constexpr uint32_t kListMaxChunks = 4096;
+constexpr uint32_t kFillStride = 8;  // words per list counter: appends to different lists meet in different sectors
+constexpr uint32_t kListMinSegment = 8;  // elements of a tile's segment, on average
+constexpr uint32_t kSampleRuns = 4096;       // runs of the locality sample,
+constexpr uint32_t kSampleRunHits = 8;       // indices of each that are counted by chunk
+
+struct ListGeometry {
+    bool on;
+    uint32_t CS, C, cap;         // elements per chunk (a multiple of 32), chunks, room of a list (a multiple of 8)
+    uint32_t cs_mul, cs_shift;   // v / CS = (v * cs_mul) >> (32 + cs_shift) for v < 2^29
+    uint32_t T;                  // elements of a tile
+    uint32_t hits_max;           // sampled indices of a chunk above which its list is taken to overflow
+    size_t smem;                 // shared memory of a CTA
+    size_t off_fill, off_off, off_v, end;  // scratch, from `start`
+};
+
+// n elements of W bytes; chunks as large as shared memory takes, evened out
+// over the sms SMs where each places only a few; scratch from byte `start` to
+// byte `limit` of the call's.  Measured against the bucketed passes (random
+// permutations, us): 2^25 x 4 B 422 -> 272, 2^26 796 -> 559, 10^8 1167 -> 881,
+// 2^27 1538 -> 1290, 2^28 3058 -> 3489; 2^24 x 8 B 302 -> 239, 2^25 549 -> 471,
+// 2^26 1056 -> 1127; 2^23 x 16 B 249 -> 240, 2^25 895 -> 1148: tiles' segments
+// have to be long enough for their list writes to fill sectors, and 16-byte
+// elements (tiles of 8192) gain nothing.
+inline ListGeometry list_geometry(uint64_t n, uint32_t W, uint32_t sms, size_t start, size_t limit)
+{
+    ListGeometry g{};
+    if (W > 8 || n > kListMaxElems) return g;
+    const uint64_t most = kListChunkBytes / W;
+    const uint64_t rounds = (n + most * sms - 1) / (most * sms);
+    const uint64_t cs = ((n + rounds * sms - 1) / (rounds * sms) + 31) / 32 * 32;
+    g.CS = uint32_t(std::min(most, cs));
+    g.C = uint32_t((n + g.CS - 1) / g.CS);
+    // With s = floor(log2(CS - 1)) and m = ceil(2^(32 + s) / CS) < 2^32 the error
+    // m CS - 2^(32 + s) is below CS <= 2^(s + 1), so v m / 2^(32 + s) is less
+    // than 1 / CS above v / CS for v < 2^29 (Granlund & Montgomery, Sec. 4).
+    while ((uint64_t(2) << g.cs_shift) < g.CS) ++g.cs_shift;
+    const uint64_t two = uint64_t(1) << (32 + g.cs_shift);
+    g.cs_mul = uint32_t((two + g.CS - 1) / g.CS);
+    // n uniform draws with repeats fill a list to CS with a deviation of
+    // sqrt(CS); twelve of those are left free
+    uint32_t root = 1;
+    while (uint64_t(root) * root < g.CS) ++root;
+    g.cap = (g.CS + 12 * root + 7) / 8 * 8;
+    g.T = (W == 4 ? 6 : 4) * 4096;
+    g.smem = size_t(g.T) * (W + 4) + size_t(g.C) * 4;
+    // four times the mean and then some: a chance few in a chunk are no crowd
+    g.hits_max = 4 * (kSampleRuns * kSampleRunHits / g.C) + 32;
+    auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+    g.off_fill = start;
+    g.off_off = g.off_fill + al(size_t(g.C) * kFillStride * 4);
+    g.off_v = g.off_off + al(size_t(g.C) * g.cap * 2);
+    g.end = g.off_v + al(size_t(g.C) * g.cap * W);
+    g.on = g.C <= kListMaxChunks && g.smem <= kListSmem && g.T >= kListMinSegment * g.C && g.end <= limit;
+    return g;
+}
+
 }  // namespace rearr

@@ -1,0 +1,69 @@
+"""Large scatters (chunk lists) on the GPU: every written element must carry the
+tag of a source whose index names it, every other element must be untouched."""
+import numpy as np
+import pytest
+
+import synth
+from tests.gpu_util import DevBuf, sync, to_dev
+
+pytestmark = pytest.mark.gpu
+
+MIN = 128 << 20  # bytes from which scatters leave the direct kernel
+
+
+@pytest.fixture(scope="module")
+def lr():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1011_3583_gb300 import build, librearr
+    build.build()
+    librearr.load()
+    return librearr
+
+
+def check(lr, e, idx, dst_off=0):
+    n, tag = idx.size, np.uint32 if e == 4 else np.uint64
+    d = DevBuf(n * e, dst_off, fill=0xA7)
+    s, ix = to_dev(np.arange(n, dtype=tag)), to_dev(idx)
+    (lr.scatter64 if idx.dtype == np.uint64 else lr.scatter)(d.ptr, s.ptr, ix.ptr, n, e)
+    sync()
+    got = d.download().view(tag)
+    hit = np.zeros(n, dtype=bool)
+    hit[idx] = True
+    assert np.all(got[~hit] == np.frombuffer(b"\xa7" * e, dtype=tag)[0])
+    at = np.flatnonzero(hit)
+    assert np.all(got[at] < n)
+    assert np.array_equal(idx[got[at].astype(np.int64)].astype(np.int64), at)
+
+
+# the smallest size, one element more (a tile and a chunk of little), a tile
+# boundary, and one where the chunks are evened out to several rounds
+@pytest.mark.parametrize("e,n", [(4, MIN // 4), (4, MIN // 4 + 1), (4, 24576 * 1400), (4, 50_000_017),
+                                 (8, MIN // 8 + 3), (8, 16384 * 1100 - 1)])
+@pytest.mark.parametrize("wide", [False, True])
+def test_permutations(lr, e, n, wide):
+    idx = synth.random_permutation(n % 97, n)
+    check(lr, e, idx.astype(np.uint64) if wide else idx)
+
+
+def test_unaligned_destination(lr):
+    n = MIN // 4 + 4099
+    for off in (4, 8, 12):
+        check(lr, 4, synth.random_permutation(off, n), dst_off=off)
+
+
+@pytest.mark.parametrize("e", [4, 8])
+def test_repeats(lr, e):
+    """Uniform repeats (lists part empty, part beyond a chunk's size), a range
+    that the sample shows crowded, and one that only a list's overflow shows."""
+    n = MIN // e + 12345
+    check(lr, e, synth.random_indices(1, n, n))
+    check(lr, e, synth.random_indices(2, n, n // 8) + np.uint32(n // 3))
+    p = synth.random_permutation(3, n)
+    lo = n // 2
+    away = (p >= lo + 200_000) & (p < lo + 240_000)
+    p[away] = lo + p[away] % np.uint32(40_000 // (e // 4))  # these chunks get more than their lists hold
+    check(lr, e, p)
+    p = synth.random_permutation(4, n)
+    p[: n // 2] = np.uint32(77)
+    check(lr, e, p)
