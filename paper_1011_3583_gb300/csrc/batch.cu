@@ -793,6 +793,11 @@ void batch_form(OpDesc &op)
         d.c_div = make_fastdiv(d.c);
         op.units = (d.n + d.unit_groups - 1) / d.unit_groups;
     }
+    if ((op.cls == OC_INTERLACE || op.cls == OC_DEINTERLACE) && op.inter.fast) {
+        op.inter.unit_groups = uint64_t(kThreads) * kInterSteps;
+        const uint64_t groups = op.inter.n * op.inter.elem_bytes / 16;
+        op.units = std::max<uint64_t>(1, (groups + op.inter.unit_groups - 1) / op.inter.unit_groups);
+    }
     if (op.cls == OC_GATHER && op.units > 0) {
         // one iteration of gather_body per unit: 4 elements x 2 groups per
         // thread (vector path) or 4 elements per thread

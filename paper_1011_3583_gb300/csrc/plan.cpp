@@ -707,6 +707,19 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     return REARR_OK;
 }
 
+// 16-byte groups per plane and unit of a fast interlace / de-interlace of k
+// planes, `bytes` in all.  Four steps of the CTA per unit left an operation of
+// 50 MB less than one wave of CTAs.  us at four, two, one: interlaced 4096^2 x
+// 3 bytes 18.5, 17.2, 16.7, 2^23 x 5 fp32 53.9, 50.7, 49.9, 2^26 x 4 fp32 313,
+// 309, 306, but 2^25 x 8 fp32 313, 313, 317; split 4096^2 x 3 bytes 17.7, 17.4,
+// 17.1, 2^23 x 6 of 2 bytes 34.6, 33.9, 34.8, and 2^26 x 4 fp32 315, 316, 325
+// (a large split writes longer runs per plane with four).
+static uint64_t inter_unit_groups(bool inter, uint32_t k, uint64_t bytes)
+{
+    const uint64_t steps = inter ? (k <= 6 ? 1 : 2) : bytes <= (uint64_t(256) << 20) ? 2 : kInterSteps;
+    return uint64_t(kThreads) * steps;
+}
+
 // Interlace: the output's fastest axis steps over k planes that are dense in
 // the input along the axis before it.  De-interlace: the mirror image, k cells
 // dense in the input, spread over k output planes dense along the output's
@@ -761,7 +774,7 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
     d.elem_bytes = uint32_t(E);
     d.fast = 1;
     const uint64_t groups = uint64_t(n) * E / 16;
-    d.unit_groups = uint64_t(kThreads) * 4;
+    d.unit_groups = inter_unit_groups(inter, uint32_t(k), uint64_t(n) * k * E * batch);
     const uint64_t upb = (groups + d.unit_groups - 1) / d.unit_groups;
     if (upb * batch >= kMaxUnits) return false;
     d.upb = make_fastdiv(uint32_t(upb));
@@ -972,7 +985,7 @@ rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, i
         const uint64_t groups = uint64_t(n) * elem_bytes / 16;
         op.word = uint32_t(elem_bytes);
         d.c = 1;
-        d.unit_groups = uint64_t(kThreads) * 4;
+        d.unit_groups = inter_unit_groups(inter, uint32_t(k), ibytes);
         op.units = std::max<uint64_t>(1, (groups + d.unit_groups - 1) / d.unit_groups);
         d.upb = make_fastdiv(0xFFFFFFFFu);
         d.b0_div = make_fastdiv(1);

@@ -28,6 +28,7 @@ constexpr int kBatchSmemBytes = kSmemBytes > kInterStageBytes
                                     ? (kSmemBytes > 2 * kTileBytes ? kSmemBytes : 2 * kTileBytes)
                                     : (kInterStageBytes > 2 * kTileBytes ? kInterStageBytes : 2 * kTileBytes);
 constexpr int kMaxRunsPerUnit = 256;            // run offsets staged in smem
+constexpr int kInterSteps = 4;                  // fast interlace: steps of the CTA per unit (large splits, batches)
 constexpr int kStridedSteps = 4;                // strided copy: thread steps per work unit
 
 // Unsigned 32-bit division by a run-time invariant divisor with one
