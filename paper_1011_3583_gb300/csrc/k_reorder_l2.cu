@@ -878,11 +878,12 @@ cudaError_t run_lists(const ScatterLists &p, bool idx64, size_t sm, unsigned sms
 {
     constexpr int NG = W == 4 ? 6 : 4;
     auto kernel = idx64 ? k_scatter_lists<W, true, NG> : k_scatter_lists<W, false, NG>;
-    cudaError_t e = opt_in(kernel, sm);
+    // the most any size takes: a call of another thread may launch in between
+    cudaError_t e = opt_in(kernel, kListSmem);
+    if (e == cudaSuccess) e = opt_in(k_scatter_place<W>, kListSmem);
     if (e != cudaSuccess) return e;
     e = pass(kernel, std::min<unsigned>(p.tiles, sms), kListThreads, sm, s, p);
     const size_t place = size_t(p.CS) * W + p.CS / 8;
-    if (e == cudaSuccess) e = opt_in(k_scatter_place<W>, place);
     if (e != cudaSuccess) return e;
     return pass(k_scatter_place<W>, std::min<unsigned>(p.C, sms), kListThreads, place, s, p);
 }

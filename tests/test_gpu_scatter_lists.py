@@ -67,3 +67,36 @@ def test_repeats(lr, e):
     p = synth.random_permutation(4, n)
     p[: n // 2] = np.uint32(77)
     check(lr, e, p)
+
+
+def test_two_threads(lr):
+    """Calls of different sizes (so of different shared-memory needs) from two
+    threads at a time."""
+    import threading
+
+    import torch
+    jobs = []
+    for n in (MIN // 4 + 77, 50_000_017):
+        idx = synth.random_permutation(n % 89, n)
+        d, s, ix = DevBuf(n * 4, fill=0xA7), to_dev(np.arange(n, dtype=np.uint32)), to_dev(idx)
+        jobs.append((n, idx, d, s, ix, torch.cuda.Stream()))
+    sync()
+    errors = []
+
+    def work(n, idx, d, s, ix, st):
+        try:
+            for _ in range(50):
+                lr.scatter(d.ptr, s.ptr, ix.ptr, n, 4, stream=st.cuda_stream)
+        except Exception as ex:  # reported by the test's thread
+            errors.append(ex)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    sync()
+    assert not errors, errors
+    for n, idx, d, s, ix, st in jobs:
+        got = d.download().view(np.uint32)
+        assert np.array_equal(idx[got], np.arange(n, dtype=np.uint32))
