@@ -21,7 +21,9 @@ namespace rearr {
 // into shared memory at addresses congruent to their global ones modulo
 // `chunk` (every shared-memory stride is congruent to its input stride), so
 // no span needs an aligned start.  A cell's place in shared memory is linear
-// in its digits.
+// in its digits.  A chunk that would reach past either end of the source (the
+// first and the last of an op whose source does not start or end on a chunk)
+// is copied cell by cell instead: nothing outside the source is read.
 constexpr int kSpanAxes = 4;        // axes of either chain
 constexpr int kSpanOuter = 8;       // unit-index digits
 constexpr int kSpanMaxSpans = 512;  // input / output spans per unit
@@ -30,7 +32,8 @@ constexpr int kSpanMaxLut = 8192;   // cells of an output span that runs over se
 
 struct SpanDesc {
     char *dst;
-    const char *src;
+    const char *src;              // the op's first cell, and
+    const char *src_end;          // the end of its last
     int64_t row_in[kSpanAxes];    // input spans: digits' input strides, fastest first
     int64_t run_out[kSpanAxes];   // output spans: digits' output strides
     int64_t uin[kSpanOuter], uout[kSpanOuter];
@@ -47,6 +50,8 @@ struct SpanDesc {
     int32_t ua, ub;
     uint32_t row_bytes_a, n_runs_a, run_cells_a;  // per index of the input chain's partial axis (0: not on it)
     uint32_t n_rows_b, run_cells_b;               // per index of the output chain's partial axis (0: not on it)
+    int64_t reach;                // bytes from a full unit's origin to its last input span's start
+    int64_t reach_b;              // of those, per index of the output chain's partial axis (0: not on it)
     uint32_t chunk;               // bytes of a copy: 16, 8 or 4
     uint32_t load_lanes, store_lanes;  // lanes a span is shared out over when it is copied / stored
     uint32_t tile_bytes;          // shared memory of the staged spans (multiple of 16)
@@ -56,6 +61,13 @@ struct SpanDesc {
     int32_t no;
     uint32_t units;
 };
+
+// Whether chunks around [src, src + bytes) of a unit reach outside the source.
+RH_HD bool span_at_edge(const SpanDesc &d, const char *src, int64_t bytes)
+{
+    const uintptr_t c = d.chunk - 1;
+    return (uintptr_t(src) & ~c) < uintptr_t(d.src) || ((uintptr_t(src) + uintptr_t(bytes) + c) & ~c) > uintptr_t(d.src_end);
+}
 
 // Shared memory of a unit: staged spans, the spans' offsets, the table of an
 // output span's cells.

@@ -61,13 +61,39 @@ struct SpanUnit {
     const char *src;
     char *dst;
     uint32_t rows, runs, row_bytes, cells;
+    bool edge;  // chunks of it reach outside the source
 };
+
+// The same for a unit at an end of the source: a chunk that reaches outside it
+// is copied cell by cell, what lies inside.  (Chunks no wider than a cell never do.)
+template <int CW, int E>
+__device__ __noinline__ void span_load_edge(uint32_t group, uint32_t lane, uint32_t groups, const SpanDesc &d,
+                                            const SpanUnit &u, unsigned char *tile, const int64_t *row_in,
+                                            const uint32_t *row_sm)
+{
+    const uint32_t base = uint32_t(reinterpret_cast<uintptr_t>(u.src) & 15);
+    for (uint32_t row = group; row < u.rows; row += groups) {
+        const uintptr_t g = reinterpret_cast<uintptr_t>(u.src) + row_in[row];
+        const uint32_t left = u.row_bytes + (uint32_t(g) & (CW - 1));
+        const char *p = reinterpret_cast<const char *>(g & ~uintptr_t(CW - 1));
+        unsigned char *t = tile + ((base + row_sm[row]) & ~uint32_t(CW - 1));
+        for (uint32_t x = lane * CW; x < left; x += d.load_lanes * CW) {
+            if (p + x >= d.src && p + x + CW <= d.src_end) {
+                cp_async<CW>(t + x, p + x);
+            } else {
+                for (uint32_t k = x; k < x + CW; k += E)
+                    if (p + k >= d.src && p + k + E <= d.src_end) sts<E>(t + k, ldg_any<E>(p + k));
+            }
+        }
+    }
+}
 
 __device__ __forceinline__ void span_unit(const SpanDesc &d, uint32_t u, SpanUnit &x)
 {
     const char *src = d.src;
     char *dst = d.dst;
     uint32_t rows = d.n_rows, runs = d.n_runs, row_bytes = d.row_bytes, cells = d.run_cells;
+    int64_t reach = d.reach;
 #pragma unroll 1
     for (int i = d.no - 1; i >= 0; --i) {
         uint32_t dig;
@@ -84,8 +110,10 @@ __device__ __forceinline__ void span_unit(const SpanDesc &d, uint32_t u, SpanUni
             const uint32_t k = min(d.kb, d.nb - dig * d.kb);
             if (d.n_rows_b) rows = k * d.n_rows_b;
             if (d.run_cells_b) cells = k * d.run_cells_b;
+            reach -= int64_t(d.kb - k) * d.reach_b;
         }
     }
+    x.edge = span_at_edge(d, src, reach + row_bytes);
     x.src = src;
     x.dst = dst;
     x.rows = rows;
@@ -178,7 +206,10 @@ __device__ __forceinline__ void span_units(const SpanDesc &d, uint32_t u0, uint3
     if (d.fixed && st.lane * V + V <= d.run_cells) span_offsets<V, LUT>(lut, st.lane * V, ch0, fixed);
     for (uint32_t u = u0; u < u1; u += u_step) {
         const SpanUnit x = unit;
-        if (d.chunk == 16) span_load<16>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
+        if (E < 16 && x.edge) {  // (`unit` still holds x)
+            if (E < 4 && d.chunk == 4) span_load_edge<4, E>(ld.group, ld.lane, ld.groups, d, unit, tile, row_in, row_sm);
+            else span_load_edge<16, E>(ld.group, ld.lane, ld.groups, d, unit, tile, row_in, row_sm);
+        } else if (d.chunk == 16) span_load<16>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
         else if (d.chunk == 8) span_load<8>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
         else span_load<4>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
         cp_async_commit();

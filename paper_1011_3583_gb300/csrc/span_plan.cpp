@@ -123,6 +123,8 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
     std::memset(&d, 0, sizeof(d));
     d.dst = dst;
     d.src = src;
+    d.src_end = src + E;
+    for (int i = 0; i < R; ++i) d.src_end += (ax[i].extent - 1) * ax[i].stride;
     d.E = uint32_t(E);
     d.row_bytes = uint32_t(c[0].run);
     d.run_cells = uint32_t(c[1].run / E);
@@ -170,6 +172,7 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
         d.row_sm[nr] = uint32_t(s);
         ++nr;
         d.n_rows *= uint32_t(K[x]);
+        d.reach += (K[x] - 1) * ax[x].stride;
         at = s * K[x];
     }
     d.tile_bytes = uint32_t((at + 32 + 15) / 16 * 16);
@@ -223,7 +226,10 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
     }
     if (part[1] >= 0 && part[1] != part[0]) {
         d.run_cells_b = uint32_t(c[1].run / E / K[part[1]]);
-        if (!on(0, part[1])) d.n_rows_b = d.n_rows / uint32_t(K[part[1]]);
+        if (!on(0, part[1])) {
+            d.n_rows_b = d.n_rows / uint32_t(K[part[1]]);
+            d.reach_b = ax[part[1]].stride;
+        }
     }
     d.no = no;
     d.units = uint32_t(units);
@@ -252,11 +258,12 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
 }
 
 // Host run of a span descriptor as the kernel walks it, checking what the
-// kernel relies on: copies aligned on both sides, inside the staged area,
-// each at an address no other span's chunk takes, holding at least one byte
-// of the span; every cell read from a byte some copy delivered; every store
-// inside the destination.
-static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, std::string &err)
+// kernel relies on: copies aligned on both sides, inside the source array and
+// the staged area, each at an address no other span's chunk takes, holding at
+// least one byte of the span; every cell read from a byte some copy delivered;
+// every store inside the destination.
+static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, const char *src0, size_t src_bytes,
+                         std::string &err)
 {
     const int E = int(d.E), cw = int(d.chunk);
     auto digits = [&](uint32_t q, const uint32_t *ext, const uint32_t *sm, const int64_t *st, int64_t &off) {
@@ -276,6 +283,7 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, std::s
         const char *src = d.src;
         char *dst = d.dst;
         uint32_t rows = d.n_rows, runs = d.n_runs, len = d.row_bytes, cells = d.run_cells, q = u;
+        int64_t reach = d.reach;
         for (int i = d.no - 1; i >= 0; --i) {
             uint32_t dig;
             fdivmod(q, d.udiv[i], q, dig);
@@ -291,8 +299,11 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, std::s
                 const uint32_t k = std::min(d.kb, d.nb - dig * d.kb);
                 if (d.n_rows_b) rows = k * d.n_rows_b;
                 if (d.run_cells_b) cells = k * d.run_cells_b;
+                reach -= int64_t(d.kb - k) * d.reach_b;
             }
         }
+        const bool edge = span_at_edge(d, src, reach + len);
+        const uintptr_t lo = uintptr_t(src0), hi = lo + src_bytes;
         std::fill(tile.begin(), tile.end(), 0xCD);
         std::fill(owner.begin(), owner.end(), -1);
         const uint32_t base = uint32_t(uintptr_t(src) & 15);
@@ -306,7 +317,10 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, std::s
                 const uint32_t at = ((base + sm) & ~uint32_t(cw - 1)) + ch * cw;
                 if ((g - (base + sm)) % uintptr_t(cw)) { err = "span: shared-memory address not congruent"; return false; }
                 if (at + cw > d.tile_bytes) { err = "span: copy outside the staged area"; return false; }
+                const bool cut = edge && (p < uintptr_t(d.src) || p + cw > uintptr_t(d.src_end));  // copied cell by cell
                 for (int k = 0; k < cw; ++k) {
+                    if (cut && (p + k < uintptr_t(d.src) || p + k >= uintptr_t(d.src_end))) continue;
+                    if (p + k < lo || p + k >= hi) { err = "span: read outside the source"; return false; }
                     if (owner[at + k] >= 0) { err = "span: two copies overlap"; return false; }
                     owner[at + k] = int(r);
                     // bytes of the chunk outside the span are whatever lies there
@@ -442,7 +456,7 @@ bool selftest_span(std::string &err)
         shared += d.ua >= 0 && d.run_cells_a;
         narrow += d.chunk < 16;
         std::memset(dst, 0, out_bytes);
-        if (!span_emulate(d, dst, out_bytes, err) || !same("the spans")) return false;
+        if (!span_emulate(d, dst, out_bytes, src, bytes, err) || !same("the spans")) return false;
     }
     if (plans < 300 || partial < 50 || luts < 50 || shared < 10 || narrow < 20 || inter < 10 || planes - inter < 10) {
         err = "span self-test planned " + std::to_string(plans) + " copies (" + std::to_string(partial) + " partial, " +
