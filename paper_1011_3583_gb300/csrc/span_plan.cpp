@@ -381,10 +381,13 @@ bool selftest_span(std::string &err)
         x ^= x << 13; x ^= x >> 7; x ^= x << 17;
         return x % n;
     };
-    int plans = 0, partial = 0, luts = 0, shared = 0, narrow = 0, planes = 0, inter = 0;
-    for (int t = 0; t < 12000 && (plans < 500 || planes < 60); ++t) {
+    int plans = 0, partial = 0, luts = 0, shared = 0, narrow = 0, planes = 0, inter = 0, full = 0;
+    for (int t = 0; t < 12000 && (plans < 500 || planes < 60 || full < 200); ++t) {
         const int rank = 2 + int(rnd(5));
         const int E = 1 << rnd(5);
+        // units as those of a batch, of 16 KB whatever the op's size, in half
+        // of the draws, on arrays that are long enough for some of them
+        const bool alone = rnd(2) == 0;
         int64_t dims[kMaxRank];
         uint64_t total = 1;
         for (int i = 0; i < rank; ++i) {
@@ -392,7 +395,7 @@ bool selftest_span(std::string &err)
             if (rnd(3) == 0) dims[i] = rnd(2) ? (dims[i] + 15) / 16 * 16 : 2 + int64_t(rnd(4));
             total *= uint64_t(dims[i]);
         }
-        if (total > (uint64_t(1) << 16) || total < 64) continue;
+        if (total > (uint64_t(1) << (alone ? 16 : 17)) || total < 64) continue;
         int perm[kMaxRank];
         for (int i = 0; i < rank; ++i) perm[i] = i;
         for (int i = rank - 1; i > 0; --i) std::swap(perm[i], perm[rnd(uint64_t(i) + 1)]);
@@ -449,19 +452,22 @@ bool selftest_span(std::string &err)
             if (!planes_emulate(op, pl, dst, out_bytes, err) || !same("interlaces")) return false;
         }
         SpanDesc d;
-        if (!plan_span(ax, E, dst, src, d)) continue;
+        if (!plan_span(ax, E, dst, src, d, alone)) continue;
         ++plans;
         partial += d.ua >= 0 || d.ub >= 0;
         luts += d.lut;
         shared += d.ua >= 0 && d.run_cells_a;
         narrow += d.chunk < 16;
+        full += uint64_t(d.n_rows) * d.row_bytes > 2 * kSpanMinBoxBytes;
         std::memset(dst, 0, out_bytes);
         if (!span_emulate(d, dst, out_bytes, src, bytes, err) || !same("the spans")) return false;
     }
-    if (plans < 300 || partial < 50 || luts < 50 || shared < 10 || narrow < 20 || inter < 10 || planes - inter < 10) {
+    if (plans < 300 || partial < 50 || luts < 50 || shared < 10 || narrow < 20 || inter < 10 || planes - inter < 10 ||
+        full < 100) {
         err = "span self-test planned " + std::to_string(plans) + " copies (" + std::to_string(partial) + " partial, " +
               std::to_string(luts) + " of several axes, " + std::to_string(shared) + " sharing a range, " +
-              std::to_string(narrow) + " in narrow copies) and " + std::to_string(planes) + " interlaces";
+              std::to_string(narrow) + " in narrow copies, " + std::to_string(full) + " of full units) and " +
+              std::to_string(planes) + " interlaces";
         return false;
     }
     return true;

@@ -58,6 +58,18 @@ def test_spans_unaligned(lr, orc, e, src_off, dst_off):
         check(lr, orc, e, dims, perm, src_off, dst_off)
 
 
+# Calls large enough (10 MB and more) to be cut into units of the full 16 KB:
+# odd planes, an odd rank-3 rotation, thin planes, a base off the grid.
+@pytest.mark.parametrize("e,dims,perm,src_off,dst_off", [
+    (1, [3331, 4099], [1, 0], 0, 0), (1, [251, 133, 517], [2, 0, 1], 3, 5), (1, [262147, 9, 7], [0, 2, 1], 1, 0),
+    (2, [2053, 4099], [1, 0], 0, 0), (2, [131, 233, 257], [2, 0, 1], 6, 2), (2, [131101, 11, 6], [0, 2, 1], 2, 4),
+    (4, [2053, 2051], [1, 0], 0, 0), (4, [131, 133, 257], [2, 0, 1], 4, 8), (4, [65543, 13, 5], [0, 2, 1], 12, 0),
+    (8, [1031, 2053], [1, 0], 8, 0)])
+def test_full_units(lr, orc, e, dims, perm, src_off, dst_off):
+    assert int(np.prod(dims)) * e > 608 * 16384
+    check(lr, orc, e, dims, perm, src_off, dst_off)
+
+
 # planes of exactly a warp's 512 bytes, one group past a unit, two batch axes,
 # k of every staging form
 @pytest.mark.parametrize("e", [1, 2, 4, 8])
