@@ -237,7 +237,7 @@ rearr_status rearr_permute_describe(size_t elem_bytes, int rank, const int64_t *
     PermPlan pl;
     std::string err;
     rearr_status st = plan_permute(reinterpret_cast<void *>(dst_addr), reinterpret_cast<const void *>(src_addr),
-                                   elem_bytes, rank, dims, perm, pl, err);
+                                   elem_bytes, rank, dims, perm, pl, err, PlanFor::kOp);
     if (st != REARR_OK) return fail(st, "rearr_permute_describe: " + err);
     *info = pl.info;
     return REARR_OK;
@@ -253,7 +253,8 @@ rearr_status rearr_reorder_nm_describe(size_t elem_bytes, int rank_in, const int
     PermPlan pl;
     std::string err;
     rearr_status st = plan_reorder_nm(reinterpret_cast<void *>(dst_addr), reinterpret_cast<const void *>(src_addr),
-                                      elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err);
+                                      elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err,
+                                      PlanFor::kOp);
     if (st != REARR_OK) return fail(st, "rearr_reorder_nm_describe: " + err);
     *info = pl.info;
     return REARR_OK;

@@ -347,7 +347,7 @@ rearr_status rearr_plan_add_permute(rearr_plan *plan, void *dst, const void *src
     if (plan->finalized) return fail(REARR_EBUSY, "rearr_plan_add_permute: plan is finalized");
     PermPlan pl;
     std::string err;
-    rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err, true);
+    rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err, PlanFor::kBatch);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_permute: " + err);
     return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
 }
@@ -372,7 +372,8 @@ rearr_status rearr_plan_add_reorder_nm(rearr_plan *plan, void *dst, const void *
     if (plan->finalized) return fail(REARR_EBUSY, "rearr_plan_add_reorder_nm: plan is finalized");
     PermPlan pl;
     std::string err;
-    rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err, true);
+    rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err,
+                                      PlanFor::kBatch);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_reorder_nm: " + err);
     return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
 }

@@ -358,7 +358,7 @@ static bool plan_box(const std::vector<Axis> &ax, int64_t E, uintptr_t da, uintp
 // given in order (slowest first) with their input byte strides; src already
 // points at the element of output index 0.  The output is contiguous.
 static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, const std::vector<Axis> &in_axes,
-                              uint64_t total, PermPlan &pl, std::string &err, bool in_batch)
+                              uint64_t total, PermPlan &pl, std::string &err, PlanFor what)
 {
     rearr_permute_info &info = pl.info;
     const uint64_t bytes = total * elem_bytes;
@@ -692,10 +692,10 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     // copy rate already, and small ones are over before a span copy has its
     // tables (1479 x 381 2-byte cells: 4.7 against 5.2 us; 1001 x 999 bytes:
     // 6.7 against 5.1).
-    if (W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
+    if (what == PlanFor::kOp || W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
     const bool sparse = op.cls == OC_TILE && 3 * n_cells < 2 * op.units * uint64_t(t.TA) * t.TB;
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
-    if (in_batch) {
+    if (what == PlanFor::kBatch) {
         pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || sparse || (op.cls == OC_TILE && narrow)) &&
                             plan_span(ax, cell, static_cast<char *>(dst), src, pl.batch_span, false);
         return REARR_OK;
@@ -783,7 +783,7 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
 }
 
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank, const int64_t *dims,
-                          const int *perm, PermPlan &pl, std::string &err, bool in_batch)
+                          const int *perm, PermPlan &pl, std::string &err, PlanFor what)
 {
     std::memset(&pl, 0, sizeof(pl));
     rearr_permute_info &info = pl.info;
@@ -825,12 +825,12 @@ rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int ran
     for (int i = rank - 2; i >= 0; --i) s[i] = s[i + 1] * dims[i + 1];
     std::vector<Axis> ax;
     for (int i = 0; i < rank; ++i) ax.push_back(Axis{dims[perm[i]], s[perm[i]]});
-    return plan_axes(dst, static_cast<const char *>(src), elem_bytes, ax, total, pl, err, in_batch);
+    return plan_axes(dst, static_cast<const char *>(src), elem_bytes, ax, total, pl, err, what);
 }
 
 rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int rank_in, const int64_t *dims,
                              int rank_out, const int *order, const int64_t *base, const int64_t *range,
-                             PermPlan &pl, std::string &err, bool in_batch)
+                             PermPlan &pl, std::string &err, PlanFor what)
 {
     std::memset(&pl, 0, sizeof(pl));
     pl.info.plane_a = -1;
@@ -880,7 +880,7 @@ rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int 
     for (int a = 0; a < rank_in; ++a) off += base[a] * s[a];
     std::vector<Axis> ax;
     for (int i = 0; i < rank_out; ++i) ax.push_back(Axis{range[order[i]], s[order[i]]});
-    return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err, in_batch);
+    return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err, what);
 }
 
 rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_t n, size_t elem_bytes,
@@ -1198,6 +1198,30 @@ static bool selftest_box(std::string &err)
     return true;
 }
 
+// The forms a permute is planned in, by what it is planned for.
+static bool selftest_plan_for(std::string &err)
+{
+    const int64_t ragged[3] = {251, 333, 517}, planes[3] = {32, 3, 65536};
+    const int rotated[3] = {2, 0, 1}, swapped[3] = {0, 2, 1};
+    void *dst = reinterpret_cast<void *>(uintptr_t(1) << 47);
+    const void *src = reinterpret_cast<const void *>(uintptr_t(1) << 46);
+    for (int i = 0; i < 6; ++i) {
+        const bool inter = i >= 3;
+        const PlanFor what[3] = {PlanFor::kCall, PlanFor::kBatch, PlanFor::kOp};
+        const PlanFor w = what[i % 3];
+        PermPlan pl;
+        if (plan_permute(dst, src, 4, 3, inter ? planes : ragged, inter ? swapped : rotated, pl, err, w) != REARR_OK)
+            return false;
+        const bool call = w == PlanFor::kCall;
+        if (pl.op.units == 0 || pl.use_planes != (call && inter) || pl.use_span != (call && !inter) ||
+            pl.use_batch_span != (w == PlanFor::kBatch)) {
+            err = "a permute is planned in forms that are not asked for";
+            return false;
+        }
+    }
+    return true;
+}
+
 bool selftest_host(std::string &err)
 {
     // Fast division against the hardware divide on divisors and dividends
@@ -1251,7 +1275,7 @@ bool selftest_host(std::string &err)
         err = "pow2_align";
         return false;
     }
-    return selftest_box(err) && selftest_span(err);
+    return selftest_box(err) && selftest_plan_for(err) && selftest_span(err);
 }
 
 }  // namespace rearr

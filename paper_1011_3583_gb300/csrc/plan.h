@@ -18,17 +18,21 @@ struct Axis {
     int64_t stride;  // input stride in bytes
 };
 
+// What a permute is planned for: a single call, an op of a captured batch, or
+// the op alone (the server's requests, the describe calls).
+enum class PlanFor { kCall, kBatch, kOp };
+
 struct PermPlan {
     rearr_permute_info info;  // what rearr_permute_describe reports
-    OpDesc op;                // descriptor of the body that runs it (in a batch, always this one)
-    // What a single call runs instead, if there is one: interlaces of a few
-    // planes, or a span copy.
+    OpDesc op;                // descriptor of the work-list body
+    // kCall: what runs instead, if there is one: interlaces of a few planes, or
+    // a span copy.
     bool use_planes, use_span;
     OpDesc planes_op;
     char *planes[kInlineK];
     SpanDesc span;
-    SpanDesc batch_span;      // the span copy a captured batch runs instead of op,
-    bool use_batch_span;      // if it was asked for and there is one
+    SpanDesc batch_span;      // kBatch: the span copy a batch large enough for a kernel
+    bool use_batch_span;      // of them runs instead of op, if there is one
 };
 
 struct InterlacePlan {
@@ -38,13 +42,12 @@ struct InterlacePlan {
 
 // Each returns REARR_OK or REARR_EINVAL (with a message in err).  A plan with
 // op.units == 0 is a no-op.
-// batch: plan for a captured batch (batch_span) instead of a single call.
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank,
                           const int64_t *dims, const int *perm, PermPlan &pl, std::string &err,
-                          bool batch = false);
+                          PlanFor what = PlanFor::kCall);
 rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int rank_in, const int64_t *dims,
                              int rank_out, const int *order, const int64_t *base, const int64_t *range,
-                             PermPlan &pl, std::string &err, bool batch = false);
+                             PermPlan &pl, std::string &err, PlanFor what = PlanFor::kCall);
 // Gather dst[i] = src[idx[i]] (or, with scatter, dst[idx[i]] = src[i]) with
 // idx_bytes-byte (4 or 8) indices.
 rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_t n,

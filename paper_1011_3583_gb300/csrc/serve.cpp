@@ -121,7 +121,7 @@ rearr_status plan_request(const Req &r, OpDesc &op, std::vector<char *> &planes,
         case REARR_OP_PERMUTE: {
             PermPlan pl;
             rearr_status st = plan_permute(reinterpret_cast<void *>(r.outs[0]), reinterpret_cast<const void *>(r.ins[0]),
-                                           s.elem_bytes, s.rank, s.dims, s.perm, pl, err);
+                                           s.elem_bytes, s.rank, s.dims, s.perm, pl, err, PlanFor::kOp);
             op = pl.op;
             return st;
         }
