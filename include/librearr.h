@@ -126,8 +126,9 @@ rearr_status rearr_reorder(void *dst, const void *src, const uint32_t *idx, size
  *   rearr_reorder (a scatter's buckets by destination chunk), with the same
  *   locality check and scratch pool.  A scatter of 4- or 8-byte elements of up
  *   to about 640 / 400 MB first sorts them into lists per shared-memory-sized
- *   destination chunk and places each list in shared memory; the passes run
- *   where a list would overflow (indices crowded in a few chunks).
+ *   destination chunk and places each list in shared memory (an element whose
+ *   list is full is stored directly); the passes run where the sample finds the
+ *   indices crowded in some chunks.
  * ------------------------------------------------------------------------- */
 rearr_status rearr_scatter(void *dst, const void *src, const uint32_t *idx, size_t n,
                            size_t elem_bytes, rearr_stream_t stream);

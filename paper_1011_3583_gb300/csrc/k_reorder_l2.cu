@@ -36,7 +36,8 @@
 // (destination index, element) pairs, and a linear pass writes
 // dst[s[k]] = v[k] with the destination chunk L2-resident.  Scatters of 4- and
 // 8-byte elements up to a size go through chunk lists first
-// (scatter_chunks.cuh) and take these passes only where a list overflows.
+// (scatter_chunks.cuh) and take these passes only where the sample finds their
+// indices crowded in some chunks.
 // Every pass is launched behind the one before (pass_enter()), which takes
 // most of the launch off those that return at once: block-shuffled 2^26 x 4 B
 // scatter 149 -> 142 us with two passes more, gather 2^25 x 4 B 338 -> 327,
@@ -98,7 +99,7 @@ struct L2Reorder {
     uint32_t tiles;                // 4096-index tiles of the sequence
     unsigned long long near_threshold;
     // a scatter tried through chunk lists first (scatter_chunks.cuh): the flag
-    // that they overflowed; their chunks and the sampled indices of each
+    // that the indices are too crowded for them; their chunks and the sampled indices of each
     const uint32_t *over;
     uint32_t *hits;
     uint32_t list_mul, list_shift, list_C;
@@ -912,7 +913,7 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // A scatter goes through chunk lists; the bucketed passes below then run
-    // only if a list overflowed, or the sample says that one would.
+    // only if the sample says that many elements would not fit them.
     const ListGeometry lg = list_geometry(g.n, W, uint32_t(sms), off_s, bytes);
     const bool lists = W <= 8 && g.scatter && lg.on &&
                        reorder_geometry(g.n, W, false, reorder_smem_max_buckets()).smem_scatter;
@@ -1013,7 +1014,8 @@ cudaError_t run_l2(const GatherDesc &g, cudaStream_t s)
         f.cs_mul = lg.cs_mul;
         f.cs_shift = lg.cs_shift;
         f.tiles = uint32_t((g.n + lg.T - 1) / lg.T);
-        f.hits_max = lg.hits_max;
+        f.hits_full = lg.hits_full;
+        f.hits_past = lg.hits_past;
         f.near = p.near;
         f.near_threshold = p.near_threshold;
         f.over = reinterpret_cast<uint32_t *>(scratch + 24);  // zeroed with the counters

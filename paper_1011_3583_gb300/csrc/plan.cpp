@@ -13,6 +13,7 @@
 //      axes with the other axes as batch (Sec. III.B: the 2-D plane of the
 //      fastest dimensions of the original and the desired order).
 #include "plan.h"
+#include "reorder_geometry.h"
 
 #include <algorithm>
 #include <cmath>
@@ -1198,6 +1199,35 @@ static bool selftest_box(std::string &err)
     return true;
 }
 
+// Geometry of the scatter's chunk lists: within the call's scratch, with room
+// for half as many elements again as a chunk has, and an exact chunk division.
+static bool selftest_lists(std::string &err)
+{
+    int on = 0;
+    for (uint32_t W : {4u, 8u})
+        for (uint32_t sms : {148u, 152u, 160u})
+            for (uint64_t n = kReorderL2MinBytes / W; n <= kListMaxElems; n += n / 7 + 3) {
+                const ReorderGeometry gm = reorder_geometry(n, W, true, kReorderMaxSmemBuckets);
+                const ListGeometry g = list_geometry(n, W, sms, gm.off_s, gm.bytes);
+                if (!g.on) continue;
+                ++on;
+                bool ok = 2 * uint64_t(g.cap) >= 3 * uint64_t(g.CS) && g.cap % 8 == 0 && g.CS % 32 == 0 &&
+                          g.end <= gm.bytes && uint64_t(g.C) * g.cap < (uint64_t(1) << 31) &&
+                          size_t(g.CS) * W + g.CS / 8 <= kListSmem;
+                for (uint64_t c = 1; c <= g.C; ++c)
+                    for (uint64_t v : {c * g.CS - 1, c * g.CS})
+                        if (v < n) ok &= (uint64_t(uint32_t(v)) * g.cs_mul >> (32 + g.cs_shift)) == v / g.CS;
+                if (!ok) {
+                    err = "chunk lists of " + std::to_string(n) + " elements of " + std::to_string(W) + " bytes: " +
+                          std::to_string(g.C) + " chunks of " + std::to_string(g.CS) + ", lists of " +
+                          std::to_string(g.cap);
+                    return false;
+                }
+            }
+    if (on < 30) err = "chunk lists planned for " + std::to_string(on) + " sizes only";
+    return on >= 30;
+}
+
 // The forms a permute is planned in, by what it is planned for.
 static bool selftest_plan_for(std::string &err)
 {
@@ -1275,7 +1305,7 @@ bool selftest_host(std::string &err)
         err = "pow2_align";
         return false;
     }
-    return selftest_box(err) && selftest_plan_for(err) && selftest_span(err);
+    return selftest_box(err) && selftest_lists(err) && selftest_plan_for(err) && selftest_span(err);
 }
 
 }  // namespace rearr

@@ -76,7 +76,8 @@ struct ListGeometry {
     uint32_t CS, C, cap;         // elements per chunk (a multiple of 32), chunks, room of a list (a multiple of 8)
     uint32_t cs_mul, cs_shift;   // v / CS = (v * cs_mul) >> (32 + cs_shift) for v < 2^29
     uint32_t T;                  // elements of a tile
-    uint32_t hits_max;           // sampled indices of a chunk above which its list is taken to overflow
+    uint32_t hits_full;          // sampled indices of a chunk that stand for a full list
+    uint32_t hits_past;          // those beyond full lists, in all, that are let through
     size_t smem;                 // shared memory of a CTA
     size_t off_fill, off_off, off_v, end;  // scratch, from `start`
 };
@@ -105,17 +106,24 @@ inline ListGeometry list_geometry(uint64_t n, uint32_t W, uint32_t sms, size_t s
     const uint64_t two = uint64_t(1) << (32 + g.cs_shift);
     g.cs_mul = uint32_t((two + g.CS - 1) / g.CS);
     // n uniform draws with repeats fill a list to CS with a deviation of
-    // sqrt(CS); twelve of those are left free
+    // sqrt(CS); at least twelve of those are left free.  Sequences that repeat
+    // more in some chunks than in others need longer lists: all the room that
+    // the call's scratch has (CS twice at 4 bytes, 1.6 times at 8).
     uint32_t root = 1;
     while (uint64_t(root) * root < g.CS) ++root;
-    g.cap = (g.CS + 12 * root + 7) / 8 * 8;
-    g.T = (W == 4 ? 6 : 4) * 4096;
-    g.smem = size_t(g.T) * (W + 4) + size_t(g.C) * 4;
-    // four times the mean and then some: a chance few in a chunk are no crowd
-    g.hits_max = 4 * (kSampleRuns * kSampleRunHits / g.C) + 32;
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
     g.off_fill = start;
     g.off_off = g.off_fill + al(size_t(g.C) * kFillStride * 4);
+    if (limit < g.off_off + 512) return g;
+    const uint64_t room = (limit - g.off_off - 512) / (uint64_t(g.C) * (2 + W));
+    g.cap = uint32_t(std::min<uint64_t>(room, 2 * uint64_t(g.CS)) / 8 * 8);
+    if (g.cap < g.CS + 12 * root) return g;
+    g.T = (W == 4 ? 6 : 4) * 4096;
+    g.smem = size_t(g.T) * (W + 4) + size_t(g.C) * 4;
+    // A sixteenth beyond full lists: what chance gives uniform draws is a tenth
+    // of that, and as many direct stores cost less than the lists gain.
+    g.hits_full = uint32_t(uint64_t(kSampleRuns) * kSampleRunHits * g.cap / n);
+    g.hits_past = kSampleRuns * kSampleRunHits / 16;
     g.off_v = g.off_off + al(size_t(g.C) * g.cap * 2);
     g.end = g.off_v + al(size_t(g.C) * g.cap * W);
     g.on = g.C <= kListMaxChunks && g.smem <= kListSmem && g.T >= kListMinSegment * g.C && g.end <= limit;

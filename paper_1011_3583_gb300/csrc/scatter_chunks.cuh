@@ -18,9 +18,11 @@
 // 905 us, lists 594 us (shared-memory wavefronts, 60 % of the pipe's cycles:
 // ranking and placing are random accesses; one CTA of 1024 threads per SM, as
 // tiles half as large at two CTAs halved the segments and took 1114 us in
-// all), place 247 us (3.8 TB/s).  A list holds CS elements and a slack that covers
-// uniformly drawn repeats; a sequence that overflows one sets a flag on which
-// the place pass returns and the bucketed passes of k_reorder_l2.cu run.
+// all), place 247 us (3.8 TB/s).  An element whose list is full is stored at
+// once to its place in the destination (which of several elements of one
+// destination stays is unspecified).  Where the sample says that many would be,
+// the lists set a flag on which the place pass returns and the bucketed passes
+// of k_reorder_l2.cu run.
 #pragma once
 
 #include "bodies.cuh"
@@ -38,10 +40,10 @@ struct ScatterLists {
     uint32_t tiles;
     unsigned long long *near;      // locality sample (k_l2_sample)
     unsigned long long near_threshold;
-    uint32_t *over;                // set when a list overflows
+    uint32_t *over;                // set when the sample shows the indices crowded
     uint32_t *fill;                // [C] elements in the lists, 32 bytes apart; beside each the
                                    // sampled indices that fall in the chunk (k_l2_sample)
-    uint32_t hits_max;             // sampled indices a chunk may have
+    uint32_t hits_full, hits_past; // sampled indices that stand for a full list; those beyond, in all, that may be
     uint16_t *off;                 // [C][cap]
     char *v;                       // [C][cap]
 };
@@ -182,22 +184,11 @@ __device__ __forceinline__ void lists_tile(const ScatterLists &p, uint32_t t, un
     }
     __syncthreads();
     {
-        uint32_t from[PER + 1];  // segment starts, before any is replaced
 #pragma unroll
-        for (int j = 0; j <= PER; ++j) from[j] = uint32_t(j) <= per && x0 + j < p.C ? cnt[x0 + j] : m;
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            if (uint32_t(j) < per && x0 + j < p.C) {
-                const bool fits = place[j] + (from[j + 1] - from[j]) <= p.cap;
-                if (!fits) *p.over = 1;
-                // a segment that does not fit is not written (its elements' places compare past the lists' end)
-                cnt[x0 + j] = fits ? (x0 + j) * p.cap + place[j] - from[j] : 0x80000000u;
-            }
-        }
+        for (int j = 0; j < PER; ++j)
+            if (uint32_t(j) < per && x0 + j < p.C) cnt[x0 + j] = (x0 + j) * p.cap + min(place[j], p.cap) - cnt[x0 + j];
     }
     __syncthreads();
-    const uint32_t end = p.C * p.cap;  // < 2^31
 #pragma unroll 4
     for (uint32_t q = threadIdx.x; q < m; q += kListThreads) {
         uint32_t v;
@@ -211,9 +202,11 @@ __device__ __forceinline__ void lists_tile(const ScatterLists &p, uint32_t t, un
             val = lds<W>(smem + size_t(q) * W);
         }
         const uint32_t c = list_of(p, v), to = cnt[c] + q;
-        if (to < end) {
+        if (to < (c + 1) * p.cap) {  // C * cap < 2^31
             p.off[to] = uint16_t(min(v - c * p.CS, p.CS - 1));
             stg<W>(p.v + uint64_t(to) * W, val);
+        } else if (v < p.n) {
+            stg<W>(p.dst + uint64_t(v) * W, val);
         }
     }
     __syncthreads();
@@ -225,12 +218,19 @@ __global__ void __launch_bounds__(kListThreads, 1) k_scatter_lists(const Scatter
     pass_enter();
     if (!lists_on(p)) return;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t warp_sums[32];
-    // A chunk that the sample already shows crowded would overflow its list:
-    // every CTA sees the same counts and leaves.
-    bool crowded = false;
-    for (uint32_t c = threadIdx.x; c < p.C; c += kListThreads) crowded |= p.fill[size_t(c) * kFillStride + 1] > p.hits_max;
-    if (__syncthreads_or(crowded)) {
+    __shared__ uint32_t warp_sums[32], past;
+    // Sampled indices beyond full lists: every CTA sees the same counts.
+    if (threadIdx.x == 0) past = 0;
+    __syncthreads();
+    uint32_t mine = 0;
+    for (uint32_t c = threadIdx.x; c < p.C; c += kListThreads) {
+        const uint32_t h = p.fill[size_t(c) * kFillStride + 1];
+        mine += h > p.hits_full ? h - p.hits_full : 0u;
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&past, mine);
+    __syncthreads();
+    if (past > p.hits_past) {
         if (threadIdx.x == 0) *p.over = 1;
         return;
     }
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kListThreads, 1) k_scatter_place(const Scatter
     const bool vec = (reinterpret_cast<uintptr_t>(p.dst) & 15) == 0;
     for (uint32_t c = blockIdx.x; c < p.C; c += gridDim.x) {
         for (uint32_t x = threadIdx.x; x < p.CS / 32; x += kListThreads) bits[x] = 0;
-        const uint32_t have = p.fill[size_t(c) * kFillStride];
+        const uint32_t have = min(p.fill[size_t(c) * kFillStride], p.cap);
         const uint16_t *off = p.off + size_t(c) * p.cap;  // cap is a multiple of 8
         const char *v = p.v + size_t(c) * p.cap * W;
         __syncthreads();

@@ -69,6 +69,27 @@ def test_repeats(lr, e):
     check(lr, e, p)
 
 
+@pytest.mark.parametrize("e", [4, 8])
+def test_crowded(lr, e):
+    """Repeats that crowd some chunks: all of them moderately (within the lists'
+    room), a few far beyond it (stored past their lists), and so many that the
+    bucketed passes run."""
+    n = MIN // e + 4321
+    g = synth.rng(e)
+    check(lr, e, synth.random_indices(1, n, n * 3 // 4))
+    p = synth.random_indices(2, n, n)
+    hot = g.random(n) < 0.02
+    p[hot] = n // 3 + p[hot] % np.uint32(3000)
+    check(lr, e, p)
+    p = synth.random_indices(3, n, n)
+    w = np.uint32(n // 1000)
+    hot = g.random(n) < 0.1
+    p[hot] = p[hot] // w // np.uint32(40) * np.uint32(40) * w + p[hot] % w
+    check(lr, e, p)
+    check(lr, e, synth.random_indices(4, n, n // 3))
+    check(lr, e, synth.random_indices(5, n, n // 2).astype(np.uint64))
+
+
 def test_two_threads(lr):
     """Calls of different sizes (so of different shared-memory needs) from two
     threads at a time."""
