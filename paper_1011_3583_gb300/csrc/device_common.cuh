@@ -152,6 +152,21 @@ __device__ __forceinline__ int tid_x()
     return t;
 }
 
+// Programmatic dependent launch.  Every single-op kernel is launched with
+// programmatic stream serialisation: when the kernel before it on the stream
+// is also one of these, it may be launched while that one drains, its CTAs
+// taking SM slots as they free up.  Each kernel therefore first waits for
+// the grid it depends on to complete and its writes to be visible
+// (griddepcontrol.wait; a no-op when nothing is pending), and then allows
+// the next kernel to launch (griddepcontrol.launch_dependents; that launch
+// happens once every CTA of this grid has started or exited).  No memory is
+// touched before the wait, so ordering on the stream is as without it.
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // First thing in a kernel launched with programmatic stream serialisation
 // behind others of its kind that do not trigger it early: its launch overlaps
 // their drain, and no memory is touched before they are complete.  (Letting

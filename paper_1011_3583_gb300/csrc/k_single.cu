@@ -12,21 +12,6 @@ namespace rearr {
 
 std::atomic<uint64_t> g_launches{0};
 
-// Programmatic dependent launch.  Every single-op kernel is launched with
-// programmatic stream serialisation: when the kernel before it on the stream
-// is also one of these, it may be launched while that one drains, its CTAs
-// taking SM slots as they free up.  Each kernel therefore first waits for
-// the grid it depends on to complete and its writes to be visible
-// (griddepcontrol.wait; a no-op when nothing is pending), and then allows
-// the next kernel to launch (griddepcontrol.launch_dependents; that launch
-// happens once every CTA of this grid has started or exited).  No memory is
-// touched before the wait, so ordering on the stream is as without it.
-__device__ __forceinline__ void pdl_enter()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 template <int E, int VIN, int VOUT, int ROWB, int TBYTES = kTileBytes>
 __global__ void __launch_bounds__(kThreads) k_tile_fast(const __grid_constant__ TileDesc d, uint32_t n)
 {
@@ -102,19 +87,8 @@ __global__ void __launch_bounds__(kThreads) k_inter_fast(const __grid_constant__
     pdl_enter();
     __shared__ __align__(16) unsigned char smem[kThreads / 32 * K * 32 * 16];
     for (uint64_t u = blockIdx.x; u < n; u += gridDim.x) {
-        uint64_t unit = u, units = n;
-        int64_t ioff = 0, poff = 0;
-        if (p.d.upb.d < n) {  // a batch of interlaces (units < 2^32)
-            uint32_t b, r, b0, b1;
-            fdivmod(uint32_t(u), p.d.upb, b, r);
-            fdivmod(b, p.d.b0_div, b1, b0);
-            unit = r;
-            units = p.d.upb.d;
-            ioff = int64_t(b0) * p.d.b_inter[0] + int64_t(b1) * p.d.b_inter[1];
-            poff = int64_t(b0) * p.d.b_plane[0] + int64_t(b1) * p.d.b_plane[1];
-        }
-        if constexpr (INTER) interlace_fast_body<E, K>(p.d, p.planes, unit, units, smem, ioff, poff);
-        else deinterlace_fast_body<E, K>(p.d, p.planes, unit, units, smem, ioff, poff);
+        if constexpr (INTER) interlace_fast_body<E, K>(p.d, p.planes, u, n, smem);
+        else deinterlace_fast_body<E, K>(p.d, p.planes, u, n, smem);
     }
 }
 

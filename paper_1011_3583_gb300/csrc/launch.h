@@ -17,12 +17,13 @@ extern std::atomic<uint64_t> g_launches;
 // pointers of an interlace / de-interlace (ignored otherwise).
 cudaError_t launch_single(const OpDesc &op, char *const *planes_all, cudaStream_t s);
 
-// A planned permute or N-to-M box as a single call: as interlaces or a span
-// copy (k_span.cu) if it has such a plan, else the kernel of its op.
+// A planned permute or N-to-M box as a single call: as interlaces (k_planes.cu)
+// or a span copy (k_span.cu) if it has such a plan, else the kernel of its op.
+cudaError_t launch_planes(const OpDesc &op, cudaStream_t s);
 cudaError_t launch_span(const SpanDesc &d, cudaStream_t s);
 inline cudaError_t launch_permute(const PermPlan &pl, cudaStream_t s)
 {
-    if (pl.use_planes) return launch_single(pl.planes_op, pl.planes, s);
+    if (pl.use_planes) return launch_planes(pl.planes_op, s);
     return pl.use_span ? launch_span(pl.span, s) : launch_single(pl.op, nullptr, s);
 }
 

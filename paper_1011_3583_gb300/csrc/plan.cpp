@@ -702,7 +702,7 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
         return REARR_OK;
     }
     pl.use_planes = (thin || narrow || sparse) &&
-                    plan_planes(ax, cell, static_cast<char *>(dst), src, pl.planes_op, pl.planes);
+                    plan_planes(ax, cell, static_cast<char *>(dst), src, pl.planes_op);
     if (!pl.use_planes && ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16))))
         pl.use_span = plan_span(ax, cell, static_cast<char *>(dst), src, pl.span);
     return REARR_OK;
@@ -725,10 +725,9 @@ static uint64_t inter_unit_groups(bool inter, uint32_t k, uint64_t bytes)
 // the input along the axis before it.  De-interlace: the mirror image, k cells
 // dense in the input, spread over k output planes dense along the output's
 // fastest axis.  The other axes (after collapsing, at most two) are a batch.
-// k_inter_fast moves 16-byte groups on both sides, so everything has to lie on
+// k_planes moves 16-byte groups on both sides, so everything has to lie on
 // 16-byte boundaries, and a plane be long enough for a warp's 32 groups.
-bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op,
-                 char *(&planes)[kInlineK])
+bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op)
 {
     const int R = int(ax.size());
     int64_t os[kMaxRank];
@@ -768,7 +767,7 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
     op.word = uint32_t(E);
     d.inter = inter ? dst : const_cast<char *>(src);
     for (int j = 0; j < kInlineK; ++j)
-        planes[j] = d.planes[j] = j < k ? (inter ? const_cast<char *>(src) : dst) + j * plane : nullptr;
+        d.planes[j] = j < k ? (inter ? const_cast<char *>(src) : dst) + j * plane : nullptr;
     d.n = uint64_t(n);
     d.k = uint32_t(k);
     d.c = 1;
@@ -988,8 +987,6 @@ rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, i
         d.c = 1;
         d.unit_groups = inter_unit_groups(inter, uint32_t(k), ibytes);
         op.units = std::max<uint64_t>(1, (groups + d.unit_groups - 1) / d.unit_groups);
-        d.upb = make_fastdiv(0xFFFFFFFFu);
-        d.b0_div = make_fastdiv(1);
     } else {
         const int W = pow2_align(align_or, elem_bytes);
         op.word = uint32_t(W);

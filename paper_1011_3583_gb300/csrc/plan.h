@@ -29,7 +29,6 @@ struct PermPlan {
     // a span copy.
     bool use_planes, use_span;
     OpDesc planes_op;
-    char *planes[kInlineK];
     SpanDesc span;
     SpanDesc batch_span;      // kBatch: the span copy a batch large enough for a kernel
     bool use_batch_span;      // of them runs instead of op, if there is one
@@ -58,8 +57,7 @@ rearr_status plan_interlace(bool inter, char *interlaced, char *const *planes, i
 
 // A permute of the canonical axes as a batch of interlaces or de-interlaces
 // (false: it is none, or not on 16-byte boundaries).
-bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op,
-                 char *(&planes)[kInlineK]);
+bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op);
 
 // Span copy of the canonical axes (output order, slowest first; input strides
 // in bytes; one E-byte word a cell): false where it does not apply.  alone: the

@@ -221,9 +221,9 @@ struct InterlaceDesc {
     uint32_t elem_bytes;
     uint64_t unit_groups;              // 16-byte groups (fast) or words (generic) per unit
     FastDiv kc_div, c_div;             // k*c and c (generic path)
-    // A permute run as interlaces (fast path): the same planes at up to two
+    // A permute run as interlaces (plan_planes): the same planes at up to two
     // batch indices, units per index upb, outer index digits b0 (inner), b1.
-    FastDiv upb, b0_div;               // upb.d >= units: one interlace
+    FastDiv upb, b0_div;
     int64_t b_inter[2], b_plane[2];    // byte strides of the digits b0, b1
 };
 

@@ -352,7 +352,7 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, const 
 }
 
 // Host run of interlaces planned for a permute: every cell of every plane.
-static bool planes_emulate(const OpDesc &op, char *const *planes, char *dst0, size_t dst_bytes, std::string &err)
+static bool planes_emulate(const OpDesc &op, char *dst0, size_t dst_bytes, std::string &err)
 {
     const InterlaceDesc &d = op.inter;
     const int E = int(d.elem_bytes);
@@ -364,7 +364,7 @@ static bool planes_emulate(const OpDesc &op, char *const *planes, char *dst0, si
         const int64_t poff = b0 * d.b_plane[0] + b1 * d.b_plane[1];
         for (uint32_t j = 0; j < d.k; ++j)
             for (uint64_t i = 0; i < d.n; ++i) {
-                char *c = iv + (i * d.k + j) * E, *pl = planes[j] + poff + i * E;
+                char *c = iv + (i * d.k + j) * E, *pl = d.planes[j] + poff + i * E;
                 char *to = op.cls == OC_INTERLACE ? c : pl;
                 if (i == 0 && (uintptr_t(iv) % 16 || uintptr_t(pl) % 16)) { err = "planes: off the 16-byte grid"; return false; }
                 if (to < dst0 || to + E > dst0 + dst_bytes) { err = "planes: store outside the destination"; return false; }
@@ -444,12 +444,11 @@ bool selftest_span(std::string &err)
             return false;
         };
         OpDesc op;
-        char *pl[kInlineK];
-        if (plan_planes(ax, E, dst, src, op, pl)) {
+        if (plan_planes(ax, E, dst, src, op)) {
             ++planes;
             inter += op.cls == OC_INTERLACE;
             std::memset(dst, 0, out_bytes);
-            if (!planes_emulate(op, pl, dst, out_bytes, err) || !same("interlaces")) return false;
+            if (!planes_emulate(op, dst, out_bytes, err) || !same("interlaces")) return false;
         }
         SpanDesc d;
         if (!plan_span(ax, E, dst, src, d, alone)) continue;
