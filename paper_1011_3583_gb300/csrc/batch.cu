@@ -349,7 +349,7 @@ rearr_status rearr_plan_add_permute(rearr_plan *plan, void *dst, const void *src
     std::string err;
     rearr_status st = plan_permute(dst, src, elem_bytes, rank, dims, perm, pl, err, PlanFor::kBatch);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_permute: " + err);
-    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
+    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.span : nullptr);
 }
 
 rearr_status rearr_plan_add_scatter(rearr_plan *plan, void *dst, const void *src, const uint32_t *idx, size_t n,
@@ -375,7 +375,7 @@ rearr_status rearr_plan_add_reorder_nm(rearr_plan *plan, void *dst, const void *
     rearr_status st = plan_reorder_nm(dst, src, elem_bytes, rank_in, dims, rank_out, order, base, range, pl, err,
                                       PlanFor::kBatch);
     if (st != REARR_OK) return fail(st, "rearr_plan_add_reorder_nm: " + err);
-    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.batch_span : nullptr);
+    return add_op(plan, pl.op, {}, pl.use_batch_span ? &pl.span : nullptr);
 }
 
 rearr_status rearr_plan_add_reorder(rearr_plan *plan, void *dst, const void *src, const uint32_t *idx, size_t n,

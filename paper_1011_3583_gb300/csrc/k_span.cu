@@ -14,7 +14,7 @@
 // 3.3 TB/s; 1-byte 31 us, 2.8 TB/s).  Units of 16 KB measured against 24 and
 // 32 KB: 68, 87, 69 us on the fp32 case, 75, 73, 76 us on 4-channel byte images.
 #include <algorithm>
-#include <mutex>
+#include <atomic>
 
 #include "launch.h"
 #include "span_body.cuh"
@@ -95,22 +95,17 @@ template <int E, bool LUT>
 cudaError_t launch_span_as(const SpanDesc &d, cudaStream_t s)
 {
     // Per device, once: the shared-memory opt-in; SM count.
-    static std::mutex mu;
-    static int sms_of[64] = {0};
+    static std::atomic<int> sms_of[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    int sms;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!sms_of[dev]) {
-            e = cudaFuncSetAttribute(k_span<E, LUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmemMax);
-            if (e != cudaSuccess) return e;
-            e = cudaDeviceGetAttribute(&sms_of[dev], cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return e;
-        }
-        sms = sms_of[dev];
+    int sms = sms_of[dev].load(std::memory_order_acquire);
+    if (!sms) {
+        e = cudaFuncSetAttribute(k_span<E, LUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmemMax);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        sms_of[dev].store(sms, std::memory_order_release);
     }
     const uint32_t smem = span_smem_bytes(d);
     const uint32_t per_sm = std::min<uint32_t>(kSpanCtas, std::max<uint32_t>(1, 227u * 1024 / (smem + 1024 + 32)));

@@ -698,7 +698,7 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
     if (what == PlanFor::kBatch) {
         pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || sparse || (op.cls == OC_TILE && narrow)) &&
-                            plan_span(ax, cell, static_cast<char *>(dst), src, pl.batch_span, false);
+                            plan_span(ax, cell, static_cast<char *>(dst), src, pl.span, false);
         return REARR_OK;
     }
     pl.use_planes = (thin || narrow || sparse) &&

@@ -30,8 +30,9 @@ struct PermPlan {
     bool use_planes, use_span;
     OpDesc planes_op;
     SpanDesc span;
-    SpanDesc batch_span;      // kBatch: the span copy a batch large enough for a kernel
-    bool use_batch_span;      // of them runs instead of op, if there is one
+    // kBatch: whether a batch large enough for a kernel of span copies runs
+    // `span` instead of op.
+    bool use_batch_span;
 };
 
 struct InterlacePlan {

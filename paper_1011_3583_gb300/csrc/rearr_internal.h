@@ -48,8 +48,7 @@ inline FastDiv make_fastdiv(uint32_t d)
 {
     FastDiv f;
     f.d = d ? d : 1;
-    uint32_t l = 0;
-    while (l < 32 && (uint64_t(1) << l) < f.d) ++l;
+    const uint32_t l = f.d > 1 ? 32u - uint32_t(__builtin_clz(f.d - 1)) : 0u;  // 2^l >= d
     f.m = uint32_t(((uint64_t(1) << 32) * ((uint64_t(1) << l) - f.d)) / f.d + 1);
     f.s1 = l < 1 ? l : 1;
     f.s2 = l > 0 ? l - 1 : 0;

@@ -240,19 +240,24 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
     const bool on_words = out_or % uint64_t(word) == 0;
     const int64_t chunks = (c[0].run - 1 + d.chunk - 1) / d.chunk + 1;
     const int64_t words = on_words ? (c[1].run + word - 1) / word : (c[1].run - 1 + word - 1) / word + 1;
-    // Lanes a span is shared out over: the fewest passes of the CTA.
-    auto lanes = [](int64_t items, int64_t spans) {
-        int64_t best = kThreads, cost = INT64_MAX;
-        for (int64_t passes = (items + kThreads - 1) / kThreads; passes <= 64; ++passes) {
-            const int64_t l = (items + passes - 1) / passes, groups = kThreads / l;
-            const int64_t steps = passes * ((spans + groups - 1) / groups);
-            if (steps < cost) { cost = steps; best = l; }
+    // Lanes a span is shared out over: the fewest steps of the CTA.
+    auto lanes = [](uint32_t items, uint32_t spans) {
+        uint32_t best = kThreads, cost = 0xFFFFFFFFu;
+        const uint32_t least = uint32_t((uint64_t(items) * spans + kThreads - 1) / kThreads);
+        for (uint32_t passes = (items + kThreads - 1) / kThreads; passes <= 64; ++passes) {
+            const uint32_t l = (items + passes - 1) / passes, groups = kThreads / l;
+            const uint32_t steps = passes * ((spans + groups - 1) / groups);
+            if (steps < cost) {
+                cost = steps;
+                best = l;
+                if (steps <= least) break;
+            }
             if (l <= 8) break;
         }
-        return uint32_t(best);
+        return best;
     };
-    d.load_lanes = lanes(chunks, d.n_rows);
-    d.store_lanes = lanes(words, d.n_runs);
+    d.load_lanes = lanes(uint32_t(chunks), d.n_rows);
+    d.store_lanes = lanes(uint32_t(words), d.n_runs);
     d.fixed = on_words && words <= int64_t(d.store_lanes);
     return true;
 }
