@@ -16,8 +16,9 @@
  * Direct ops: where the GPU reaches host memory through the host's own page
  * tables (a coherent link such as NVLink-C2C; the pipeline's default there),
  * a permute, interlace or de-interlace whose host buffers are page-locked and
- * whose plan streams through them (copy, tiles, runs, boxes, interlace
- * kernels) runs its kernel on the host buffers directly, with no staging:
+ * whose plan streams through them (copy, tiles, runs, boxes by
+ * rearr_permute_describe; interlaces) runs that kernel on the host buffers
+ * directly, with no staging:
  * every byte still crosses the host link once, but reads and writes share it
  * in both directions inside one kernel.  Other ops, and every op on pageable
  * memory, are staged as above.  A direct op starts after everything

@@ -72,9 +72,11 @@ struct HostOut {
     size_t bytes;
 };
 
-// Device addresses of an op's inputs and outputs inside one slot.
+// Device addresses of an op's inputs and outputs, inside one slot or (on_host)
+// those of the host buffers themselves.
 struct SlotLayout {
     std::vector<char *> in, out;
+    bool on_host = false;
 };
 
 rearr_status layout(rearr_pipeline *p, int slot, const std::vector<HostRange> &ins,
@@ -102,6 +104,7 @@ rearr_status layout(rearr_pipeline *p, int slot, const std::vector<HostRange> &i
 // ends in page-locked host memory the device can address.
 bool device_views(const std::vector<HostRange> &ins, const std::vector<HostOut> &outs, SlotLayout &lay)
 {
+    lay.on_host = true;
     auto view = [](const void *h, size_t bytes, char *&d) {
         if (bytes == 0) {
             d = nullptr;
@@ -133,6 +136,10 @@ bool device_views(const std::vector<HostRange> &ins, const std::vector<HostOut> 
 
 // Plans whose kernels stream through their buffers (every byte read and
 // written about once, in runs): the ones a direct op may run on host memory.
+// A permute runs the kernel of this class there, not the span copy that takes
+// its place in device memory: over the host link the span copy's shorter runs
+// cost more than wider accesses gain (251 x 333 x 217 of 8 bytes in order
+// 2,0,1: 1162 us as tiles, 1761 as spans; 251 x 333 x 517 fp32 1619, 1931).
 bool streams(uint32_t cls)
 {
     return cls == OC_COPY || cls == OC_TILE || cls == OC_TILE_CELLS || cls == OC_RUNS || cls == OC_BOX ||
@@ -301,7 +308,8 @@ rearr_status rearr_pipeline_permute(rearr_pipeline *pipe, void *dst, const void 
     return run_op(pipe, "rearr_pipeline_permute", {{src, bytes}}, {{dst, bytes}},
                   [&](const SlotLayout &l, std::function<cudaError_t(cudaStream_t)> &go, std::string &err, uint32_t &cls) {
                       auto pl = std::make_shared<PermPlan>();
-                      rearr_status st = plan_permute(l.out[0], l.in[0], elem_bytes, rank, dims, perm, *pl, err);
+                      rearr_status st = plan_permute(l.out[0], l.in[0], elem_bytes, rank, dims, perm, *pl, err,
+                                                     l.on_host ? PlanFor::kOp : PlanFor::kCall);
                       cls = pl->info.kind == REARR_KIND_NOOP ? uint32_t(OC_COPY) : pl->op.cls;
                       go = [pl](cudaStream_t s) { return launch_permute(*pl, s); };
                       return st;

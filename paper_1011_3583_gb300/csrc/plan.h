@@ -19,7 +19,8 @@ struct Axis {
 };
 
 // What a permute is planned for: a single call, an op of a captured batch, or
-// the op alone (the server's requests, the describe calls).
+// the op alone (the server's requests, a pipeline's direct ops, the describe
+// calls).
 enum class PlanFor { kCall, kBatch, kOp };
 
 struct PermPlan {
