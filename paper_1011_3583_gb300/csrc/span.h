@@ -38,9 +38,10 @@ struct SpanDesc {
     int64_t run_out[kSpanAxes];   // output spans: digits' output strides
     int64_t uin[kSpanOuter], uout[kSpanOuter];
     FastDiv udiv[kSpanOuter];     // unit-index digits, innermost last
-    uint32_t row_ext[kSpanAxes], row_sm[kSpanAxes];  // extents and shared-memory strides
-    uint32_t run_ext[kSpanAxes], run_sm[kSpanAxes];
-    uint32_t ch_ext[kSpanAxes], ch_sm[kSpanAxes];    // the output chain's axes
+    FastDiv row_ext[kSpanAxes], run_ext[kSpanAxes];  // extents
+    uint32_t row_sm[kSpanAxes], run_sm[kSpanAxes];   // shared-memory strides
+    FastDiv ch_ext[kSpanAxes];                       // the output chain's axes,
+    uint32_t ch_sm[kSpanAxes], ch_step[kSpanAxes];   // and the digits of kThreads over them
     uint32_t n_rows, n_runs;      // spans of a full unit
     uint32_t row_bytes;           // bytes of a full input span
     uint32_t run_cells;           // cells of a full output span
@@ -53,7 +54,7 @@ struct SpanDesc {
     int64_t reach;                // bytes from a full unit's origin to its last input span's start
     int64_t reach_b;              // of those, per index of the output chain's partial axis (0: not on it)
     uint32_t chunk;               // bytes of a copy: 16, 8 or 4
-    uint32_t load_lanes, store_lanes;  // lanes a span is shared out over when it is copied / stored
+    FastDiv load_lanes, store_lanes;  // lanes a span is shared out over when it is copied / stored
     uint32_t tile_bytes;          // shared memory of the staged spans (multiple of 16)
     uint32_t lut;                 // 1: the output chain has several axes (offsets from a table)
     uint32_t fixed;               // 1: every output span starts on a word boundary and fits one pass of the lanes

@@ -12,11 +12,10 @@ namespace rearr {
 // instruction covers neighbouring chunks (words) of one or a few spans.
 struct SpanShare {
     uint32_t group, lane, groups;
-    __device__ __forceinline__ explicit SpanShare(uint32_t lanes)
+    __device__ __forceinline__ explicit SpanShare(const FastDiv &lanes)
     {
-        groups = kThreads / lanes;
-        group = threadIdx.x / lanes;
-        lane = threadIdx.x - group * lanes;
+        groups = fdiv(kThreads, lanes);
+        fdivmod(threadIdx.x, lanes, group, lane);
         if (group >= groups) group = 0xFFFFFFFFu / 2;  // past any span
     }
 };
@@ -40,16 +39,16 @@ __device__ __forceinline__ void span_load(const SpanShare &sh, uint32_t lanes, c
 }
 
 // Spans' offsets from their digits, fastest first.
-__device__ __forceinline__ void span_digits(uint32_t q, const uint32_t *ext, const int64_t *stride, const uint32_t *sms,
+__device__ __forceinline__ void span_digits(uint32_t q, const FastDiv *ext, const int64_t *stride, const uint32_t *sms,
                                             int64_t &off, uint32_t &sm)
 {
     off = 0;
     sm = 0;
 #pragma unroll
     for (int i = 0; i < kSpanAxes; ++i) {
-        if (ext[i] == 1) continue;
-        const uint32_t n = q / ext[i], dig = q - n * ext[i];
-        q = n;
+        if (ext[i].d == 1) continue;
+        uint32_t dig;
+        fdivmod(q, ext[i], q, dig);
         off += int64_t(dig) * stride[i];
         sm += dig * sms[i];
     }
@@ -77,7 +76,7 @@ __device__ __noinline__ void span_load_edge(uint32_t group, uint32_t lane, uint3
         const uint32_t left = u.row_bytes + (uint32_t(g) & (CW - 1));
         const char *p = reinterpret_cast<const char *>(g & ~uintptr_t(CW - 1));
         unsigned char *t = tile + ((base + row_sm[row]) & ~uint32_t(CW - 1));
-        for (uint32_t x = lane * CW; x < left; x += d.load_lanes * CW) {
+        for (uint32_t x = lane * CW; x < left; x += d.load_lanes.d * CW) {
             if (p + x >= d.src && p + x + CW <= d.src_end) {
                 cp_async<CW>(t + x, p + x);
             } else {
@@ -177,14 +176,13 @@ __device__ __forceinline__ void span_units(const SpanDesc &d, uint32_t u0, uint3
         span_digits(r, d.run_ext, d.run_out, d.run_sm, run_out[r], run_sm[r]);
     if constexpr (LUT) {
         // a thread's entries are kThreads apart: one decomposition, then steps with carries
-        uint32_t dig[kSpanAxes], step[kSpanAxes], ext[kSpanAxes], q = threadIdx.x, e = kThreads;
+        uint32_t dig[kSpanAxes], step[kSpanAxes], ext[kSpanAxes], q = threadIdx.x;
 #pragma unroll
         for (int i = 0; i < kSpanAxes; ++i) {
-            ext[i] = d.ch_ext[i];
-            dig[i] = ext[i] > 1 ? q % ext[i] : 0;
-            step[i] = ext[i] > 1 ? e % ext[i] : 0;
-            q = ext[i] > 1 ? q / ext[i] : q;
-            e = ext[i] > 1 ? e / ext[i] : e;
+            ext[i] = d.ch_ext[i].d;
+            step[i] = d.ch_step[i];
+            dig[i] = 0;
+            if (ext[i] > 1) fdivmod(q, d.ch_ext[i], q, dig[i]);
         }
         for (uint32_t p = threadIdx.x; p < d.run_cells; p += kThreads) {
             uint32_t sm = 0;
@@ -209,9 +207,9 @@ __device__ __forceinline__ void span_units(const SpanDesc &d, uint32_t u0, uint3
         if (E < 16 && x.edge) {  // (`unit` still holds x)
             if (E < 4 && d.chunk == 4) span_load_edge<4, E>(ld.group, ld.lane, ld.groups, d, unit, tile, row_in, row_sm);
             else span_load_edge<16, E>(ld.group, ld.lane, ld.groups, d, unit, tile, row_in, row_sm);
-        } else if (d.chunk == 16) span_load<16>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
-        else if (d.chunk == 8) span_load<8>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
-        else span_load<4>(ld, d.load_lanes, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
+        } else if (d.chunk == 16) span_load<16>(ld, d.load_lanes.d, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
+        else if (d.chunk == 8) span_load<8>(ld, d.load_lanes.d, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
+        else span_load<4>(ld, d.load_lanes.d, x.src, x.rows, x.row_bytes, tile, row_in, row_sm);
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
@@ -232,7 +230,7 @@ __device__ __forceinline__ void span_units(const SpanDesc &d, uint32_t u0, uint3
                 const unsigned char *s = cells0 + run_sm[run];
                 const uint32_t head = V > 1 ? (uint32_t(reinterpret_cast<uintptr_t>(o)) & 3) / E : 0;
 #pragma unroll 4
-                for (uint32_t w = st.lane; w * V < cells + head; w += d.store_lanes) {
+                for (uint32_t w = st.lane; w * V < cells + head; w += d.store_lanes.d) {
                     const int32_t p = int32_t(w * V) - int32_t(head);
                     if (p >= 0 && uint32_t(p) + V <= cells) {
                         uint32_t f[V];

@@ -13,6 +13,7 @@ namespace {
 constexpr uint64_t kSpanBoxBytes = 16384;    // payload of a unit of a large op
 constexpr uint64_t kSpanMinBoxBytes = 4096;  // and of a small one, so that it still fills the GPU
 constexpr uint64_t kSpanFillUnits = 608;     // units wanted: four per SM
+const FastDiv kOne = make_fastdiv(1);
 
 struct Chain {
     int ax[kSpanAxes];
@@ -129,7 +130,7 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
     d.row_bytes = uint32_t(c[0].run);
     d.run_cells = uint32_t(c[1].run / E);
     d.n_rows = d.n_runs = 1;
-    for (int i = 0; i < kSpanAxes; ++i) d.row_ext[i] = d.run_ext[i] = d.ch_ext[i] = 1;
+    for (int i = 0; i < kSpanAxes; ++i) d.row_ext[i] = d.run_ext[i] = d.ch_ext[i] = kOne;
     auto on = [&](int s, int x) {
         for (int j = 0; j < c[s].n; ++j)
             if (c[s].ax[j] == x) return true;
@@ -167,7 +168,7 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
             s = best;
         }
         sm[x] = s;
-        d.row_ext[nr] = uint32_t(K[x]);
+        d.row_ext[nr] = make_fastdiv(uint32_t(K[x]));
         d.row_in[nr] = ax[x].stride;
         d.row_sm[nr] = uint32_t(s);
         ++nr;
@@ -181,18 +182,21 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
     for (int j = 0; j < c[0].n; ++j) {
         const int x = c[0].ax[j];
         if (on(1, x)) continue;
-        d.run_ext[nu] = uint32_t(K[x]);
+        d.run_ext[nu] = make_fastdiv(uint32_t(K[x]));
         d.run_out[nu] = os[x];
         d.run_sm[nu] = uint32_t(sm[x]);
         ++nu;
         d.n_runs *= uint32_t(K[x]);
     }
     if (d.n_rows > uint32_t(kSpanMaxSpans) || d.n_runs > uint32_t(kSpanMaxSpans)) return false;
-    for (int j = 0; j < c[1].n; ++j) {
-        d.ch_ext[j] = uint32_t(K[c[1].ax[j]]);
-        d.ch_sm[j] = uint32_t(sm[c[1].ax[j]]);
-    }
     d.lut = c[1].n > 1;
+    uint32_t step = kThreads;
+    for (int j = 0; j < c[1].n; ++j) {
+        d.ch_sm[j] = uint32_t(sm[c[1].ax[j]]);
+        if (!d.lut) continue;
+        d.ch_ext[j] = make_fastdiv(uint32_t(K[c[1].ax[j]]));
+        fdivmod(step, d.ch_ext[j], step, d.ch_step[j]);
+    }
     if (d.lut && d.run_cells > uint32_t(kSpanMaxLut)) return false;
     // Unit index: the input chain's range innermost, then the output chain's,
     // then the other axes in output order.
@@ -256,9 +260,9 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
         }
         return best;
     };
-    d.load_lanes = lanes(uint32_t(chunks), d.n_rows);
-    d.store_lanes = lanes(uint32_t(words), d.n_runs);
-    d.fixed = on_words && words <= int64_t(d.store_lanes);
+    d.load_lanes = make_fastdiv(lanes(uint32_t(chunks), d.n_rows));
+    d.store_lanes = make_fastdiv(lanes(uint32_t(words), d.n_runs));
+    d.fixed = on_words && words <= int64_t(d.store_lanes.d);
     return true;
 }
 
@@ -271,12 +275,12 @@ static bool span_emulate(const SpanDesc &d, char *dst0, size_t dst_bytes, const 
                          std::string &err)
 {
     const int E = int(d.E), cw = int(d.chunk);
-    auto digits = [&](uint32_t q, const uint32_t *ext, const uint32_t *sm, const int64_t *st, int64_t &off) {
+    auto digits = [&](uint32_t q, const FastDiv *ext, const uint32_t *sm, const int64_t *st, int64_t &off) {
         uint32_t s = 0;
         off = 0;
         for (int i = 0; i < kSpanAxes; ++i) {
-            const uint32_t dig = q % ext[i];
-            q /= ext[i];
+            const uint32_t dig = q % ext[i].d;
+            q /= ext[i].d;
             s += dig * sm[i];
             if (st) off += int64_t(dig) * st[i];
         }
