@@ -34,6 +34,7 @@ constexpr uint64_t kReorderL2MinBytes = uint64_t(128) << 20;  // reorder sources
 constexpr uint64_t kMaxUnits = 0xFFFFFFFFull;
 constexpr uint64_t kGatherStepMax = uint64_t(1) << 23;  // index sequences cut into single steps
 constexpr uint64_t kSpanMinCells = uint64_t(3) << 18;  // smaller thin-plane ops stay strided copies
+constexpr uint64_t kSpanLutCells = uint64_t(12) << 20; // thin planes whose spans need a table: see span_thin()
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t &out)
 {
@@ -353,6 +354,24 @@ static bool plan_box(const std::vector<Axis> &ax, int64_t E, uintptr_t da, uintp
     info.wide_a = info.wide_b = -1;
     info.n_tiles = int64_t(units);
     return true;
+}
+
+// Whether a thin plane's span copy beats its strided copy (us, strided against
+// span).  Output spans over several axes take their offsets from a table and
+// their words one by one: that pays where every span fits one pass of the lanes
+// on word boundaries (fixed), or from kSpanLutCells cells on, several units per
+// CTA (1 byte: 9 x 3 x 340 x 1550 in order 0,2,3,1 18.3, 13.0, but 18 x 2 x 193
+// x 597 7.0, 8.0; 2 bytes: 34 x 3 x 372 x 511 24.4, 17.6, but 36 x 6 x 557 x 35
+// 6.8, 9.5; 4 bytes: 12 x 2 x 363 x 273 4.3, 6.0, 57 x 4 x 151 x 829 39.2, 39.4).
+// A span of 32 words or more whose words all lie in one bank takes a cycle a
+// lane (4 x 1168 x 2416 bytes reversed 43.7, 51.5).  Taking every third 4-byte
+// cell apart is near the copy rate either way (1817 x 1490 x 3 10.3, 12.4),
+// every fourth is not (28 x 31 x 1218 x 4 11.1, 7.2).
+static bool span_thin(const SpanDesc &d, bool lut)
+{
+    if (d.lut && !d.fixed) return lut;
+    if (d.lut) return d.store_lanes.d < 32 || d.ch_sm[0] * (4 / d.E) % 128 != 0;
+    return d.E < 4 || d.ch_sm[0] >= 16;
 }
 
 // Plans a gather of `total` elements of elem_bytes whose output axes are
@@ -683,28 +702,39 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     // NHWC, against the strided copy: 1-byte cells 106 -> 32 us, 2-byte 111 ->
     // 61, 4-byte 138 -> 119; 2^20-odd cells of 8 bytes in short planes gain
     // nothing below kSpanMinCells.
-    // Span copies, against what else ran: tiles off the 16-byte grid
-    // (251 x 333 x 517 in order 2,0,1: 1-byte cells 112 -> 31 us, 2-byte 139 ->
-    // 52, 4-byte 150 -> 68, 8-byte 136 -> 120; with 16-byte loads an 8-byte tile
-    // is as fast: 23 against 28 us for 381 x 22 x 16 x 72 reversed in pairs),
-    // tiles less than two thirds full (32 x 16 x 4 x 3520 x 4 fp32 in order
-    // 1,0,4,2,3: 219 -> 38 us), and thin planes of 1- to 4-byte cells (2^22 x 9
-    // x 7 bytes: 344 -> 154 us).  Strided copies of 8 and 16 bytes run at the
-    // copy rate already, and small ones are over before a span copy has its
-    // tables (1479 x 381 2-byte cells: 4.7 against 5.2 us; 1001 x 999 bytes:
-    // 6.7 against 5.1).
+    // Span copies, against what else ran (measured on 510 random permutes of
+    // 0.1 to 256 MB whose op is such a tile or a thin plane):
+    // - tiles without 16-byte loads: 1.1 to 25 times as fast at any fill
+    //   (251 x 333 x 517 in order 2,0,1: 1-byte cells 112 -> 31 us, 2-byte 139
+    //   -> 52, 4-byte 150 -> 68, 8-byte 136 -> 120).  Tiles with 16-byte loads
+    //   and narrower stores are faster than spans as long as they are full
+    //   enough (4-byte cells, tiles a half to full 0.35 to 0.96; 1-byte ones
+    //   three eighths full 0.33), so the line is a fill below which spans won
+    //   at each cell size (32 x 16 x 4 x 3520 x 4 fp32 in order 1,0,4,2,3: 219
+    //   -> 38 us at 6 %).
+    // - thin planes of 1- to 4-byte cells from kSpanMinCells on, by span_thin().
+    //   Strided copies of 8 and 16 bytes run at the copy rate already, and
+    //   smaller ones are over before a span copy has its tables (1479 x 381
+    //   2-byte cells: 4.7 against 5.2 us; 1001 x 999 bytes: 6.7 against 5.1).
     if (what == PlanFor::kOp || W != cell || op.cls == OC_BOX || tile_vector_bytes() != 16) return REARR_OK;
-    const bool sparse = op.cls == OC_TILE && 3 * n_cells < 2 * op.units * uint64_t(t.TA) * t.TB;
+    const bool tile = op.cls == OC_TILE;
+    const uint64_t held = op.units * uint64_t(t.TA) * t.TB;  // cells of full tiles
+    const uint64_t least_fill = cell == 1 ? 12 : cell == 2 ? 33 : cell == 4 ? 40 : 45;  // per cent
+    const bool span_tile = tile && (vin < 16 || 100 * n_cells < least_fill * held);
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
+    char *d = static_cast<char *>(dst);
     if (what == PlanFor::kBatch) {
-        pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || sparse || (op.cls == OC_TILE && narrow)) &&
-                            plan_span(ax, cell, static_cast<char *>(dst), src, pl.span, false);
+        pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || span_tile) && plan_span(ax, cell, d, src, pl.span, false);
         return REARR_OK;
     }
-    pl.use_planes = (thin || narrow || sparse) &&
-                    plan_planes(ax, cell, static_cast<char *>(dst), src, pl.planes_op);
-    if (!pl.use_planes && ((thin && cell < 8) || sparse || (op.cls == OC_TILE && narrow && (cell < 8 || vin < 16))))
-        pl.use_span = plan_span(ax, cell, static_cast<char *>(dst), src, pl.span);
+    pl.use_planes = (thin || narrow || (tile && 3 * n_cells < 2 * held)) && plan_planes(ax, cell, d, src, pl.planes_op);
+    if (pl.use_planes) return REARR_OK;
+    if (span_tile) {
+        pl.use_span = plan_span(ax, cell, d, src, pl.span);
+    } else if (thin && (cell < 4 || (cell == 4 && ax.back().extent >= 32))) {
+        const bool lut = cell < 4 && n_cells >= kSpanLutCells;
+        pl.use_span = plan_span(ax, cell, d, src, pl.span, true, lut) && span_thin(pl.span, lut);
+    }
     return REARR_OK;
 }
 
@@ -1249,6 +1279,51 @@ static bool selftest_plan_for(std::string &err)
     return true;
 }
 
+// Routes of single calls on either side of the lines drawn in plan_axes():
+// what: 0 the op itself, 1 a span copy, 2 interlaces.
+static bool selftest_routes(std::string &err)
+{
+    struct Case {
+        int what, elem, rank;
+        int64_t dims[4];
+        int perm[4];
+    };
+    static const Case cases[] = {
+        {1, 4, 3, {251, 333, 517}, {2, 0, 1}},        // tiles without 16-byte loads
+        {1, 1, 3, {2027, 37, 630}, {0, 2, 1}},
+        {1, 4, 4, {8, 441, 1247, 8}, {0, 3, 1, 2}},   // tiles an eighth full
+        {0, 1, 4, {4, 416, 1600, 48}, {0, 3, 1, 2}},  // tiles with 16-byte loads, three eighths to half full
+        {0, 2, 3, {1056, 1328, 32}, {0, 2, 1}},
+        {0, 4, 3, {258, 134, 648}, {0, 2, 1}},
+        {0, 4, 3, {243, 418, 100}, {0, 2, 1}},        // full ones
+        {0, 2, 3, {791, 61, 408}, {0, 2, 1}},
+        {1, 4, 4, {28, 31, 1218, 4}, {0, 3, 1, 2}},   // thin planes, spans along one axis
+        {0, 4, 3, {1817, 1490, 3}, {0, 2, 1}},
+        {1, 2, 4, {15, 263, 204, 3}, {0, 3, 1, 2}},
+        {1, 1, 4, {9, 3, 340, 1550}, {0, 2, 3, 1}},   // along several: enough cells
+        {1, 2, 4, {34, 3, 372, 511}, {0, 2, 3, 1}},
+        {0, 1, 4, {18, 2, 193, 597}, {0, 2, 3, 1}},   // too few
+        {0, 2, 4, {36, 6, 557, 35}, {0, 2, 3, 1}},
+        {0, 4, 4, {12, 2, 363, 273}, {0, 2, 3, 1}},   // 4-byte cells
+        {0, 1, 3, {4, 1168, 2416}, {2, 1, 0}},        // words of a span in one bank
+        {2, 1, 4, {32, 3, 1024, 1024}, {0, 2, 3, 1}},
+        {2, 2, 4, {32, 1024, 1024, 3}, {0, 3, 1, 2}},
+    };
+    for (const Case &c : cases) {
+        PermPlan pl;
+        if (plan_permute(reinterpret_cast<void *>(uintptr_t(1) << 47), reinterpret_cast<const void *>(uintptr_t(1) << 46),
+                         size_t(c.elem), c.rank, c.dims, c.perm, pl, err) != REARR_OK)
+            return false;
+        const int got = pl.use_planes ? 2 : pl.use_span ? 1 : 0;
+        if (got != c.what) {
+            err = "route " + std::to_string(got) + " instead of " + std::to_string(c.what) + " for " +
+                  std::to_string(c.dims[0]) + " x " + std::to_string(c.dims[1]) + " ... of " + std::to_string(c.elem) + " bytes";
+            return false;
+        }
+    }
+    return true;
+}
+
 bool selftest_host(std::string &err)
 {
     // Fast division against the hardware divide on divisors and dividends
@@ -1302,7 +1377,7 @@ bool selftest_host(std::string &err)
         err = "pow2_align";
         return false;
     }
-    return selftest_box(err) && selftest_lists(err) && selftest_plan_for(err) && selftest_span(err);
+    return selftest_box(err) && selftest_lists(err) && selftest_plan_for(err) && selftest_routes(err) && selftest_span(err);
 }
 
 }  // namespace rearr

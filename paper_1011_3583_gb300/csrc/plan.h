@@ -63,8 +63,10 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
 
 // Span copy of the canonical axes (output order, slowest first; input strides
 // in bytes; one E-byte word a cell): false where it does not apply.  alone: the
-// op has the GPU to itself, so a small one is cut into units that fill it.
-bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone = true);
+// op has the GPU to itself, so a small one is cut into units that fill it.  lut:
+// output spans over several axes may be longer than one pass of the lanes.
+bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone = true,
+               bool lut = true);
 
 // A fast tile planned with the 32 KB payload re-planned with the 16 KB tile of
 // the same row length (the batched kernel holds two 16 KB tiles per CTA).

@@ -24,7 +24,7 @@ struct Chain {
 
 }  // namespace
 
-bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone)
+bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, SpanDesc &d, bool alone, bool lut)
 {
     const int R = int(ax.size());
     if (R > kMaxRank || R < 2) return false;
@@ -120,6 +120,7 @@ bool plan_span(const std::vector<Axis> &ax, int64_t E, char *dst, const char *sr
         K[x] = k;
     }
     if (c[0].run < 32 || c[1].run < 32) return false;  // spans under a sector: nothing is gained by staging
+    if (!lut && c[1].n > 1 && c[1].run > kThreads * std::max<int64_t>(4, E)) return false;
 
     std::memset(&d, 0, sizeof(d));
     d.dst = dst;
