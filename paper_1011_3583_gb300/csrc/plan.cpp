@@ -34,6 +34,7 @@ constexpr uint64_t kReorderL2MinBytes = uint64_t(128) << 20;  // reorder sources
 constexpr uint64_t kMaxUnits = 0xFFFFFFFFull;
 constexpr uint64_t kGatherStepMax = uint64_t(1) << 23;  // index sequences cut into single steps
 constexpr uint64_t kSpanMinCells = uint64_t(3) << 18;  // smaller thin-plane ops stay strided copies
+constexpr int64_t kPlaneMinCells = 576;  // shorter planes are no interlaces: see plan_planes()
 constexpr uint64_t kSpanLutCells = uint64_t(12) << 20; // thin planes whose spans need a table: see span_thin()
 
 bool mul_overflows(uint64_t a, uint64_t b, uint64_t &out)
@@ -756,7 +757,12 @@ static uint64_t inter_unit_groups(bool inter, uint32_t k, uint64_t bytes)
 // dense in the input, spread over k output planes dense along the output's
 // fastest axis.  The other axes (after collapsing, at most two) are a batch.
 // k_planes moves 16-byte groups on both sides, so everything has to lie on
-// 16-byte boundaries, and a plane be long enough for a warp's 32 groups.
+// 16-byte boundaries, and a CTA works on one batch index at a time, so planes
+// have to be long (20 MB, us, strided copies against interlaces: 2 planes of
+// 128 fp32 7.2, 21.3, of 228 7.2, 12.5, of 336 7.2, 9.2; split into 6 of 64
+// 8-byte cells 6.8, 19.8, of 168 7.2, 9.1; 2 of 256 2-byte cells 11.4, 21.2, of
+// 456 11.4, 12.5; 8 of 512 bytes 17.4, 18.7).  From kPlaneMinCells cells on
+// planes of 1 to 4 bytes won by 1.03 to 5 times, of 8 bytes by 0.9 to 2.3.
 bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *src, OpDesc &op)
 {
     const int R = int(ax.size());
@@ -777,7 +783,7 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
     if (R > 4) return false;
     const int64_t k = ax[ik].extent, n = ax[ip].extent;
     const int64_t plane = inter ? ax[ik].stride : os[ik];
-    if (n * E < 512 || (n * E) % 16 != 0) return false;
+    if (n < kPlaneMinCells || (n * E) % 16 != 0) return false;
     std::memset(&op, 0, sizeof(op));
     InterlaceDesc &d = op.inter;
     uint64_t align = uint64_t(uintptr_t(dst)) | uint64_t(uintptr_t(src)) | uint64_t(plane), batch = 1;
@@ -1306,6 +1312,9 @@ static bool selftest_routes(std::string &err)
         {0, 2, 4, {36, 6, 557, 35}, {0, 2, 3, 1}},
         {0, 4, 4, {12, 2, 363, 273}, {0, 2, 3, 1}},   // 4-byte cells
         {0, 1, 3, {4, 1168, 2416}, {2, 1, 0}},        // words of a span in one bank
+        {0, 4, 3, {20480, 2, 128}, {0, 2, 1}},        // short planes
+        {0, 8, 3, {6826, 64, 6}, {0, 2, 1}},
+        {2, 4, 3, {2048, 3, 1024}, {0, 2, 1}},        // long ones
         {2, 1, 4, {32, 3, 1024, 1024}, {0, 2, 3, 1}},
         {2, 2, 4, {32, 1024, 1024, 3}, {0, 3, 1, 2}},
     };

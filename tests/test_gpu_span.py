@@ -70,12 +70,12 @@ def test_full_units(lr, orc, e, dims, perm, src_off, dst_off):
     check(lr, orc, e, dims, perm, src_off, dst_off)
 
 
-# planes of exactly a warp's 512 bytes, one group past a unit, two batch axes,
-# k of every staging form
+# planes of few groups (576 cells, the fewest) and of one past a unit, two batch
+# axes, k of every staging form
 @pytest.mark.parametrize("e", [1, 2, 4, 8])
 @pytest.mark.parametrize("k", [2, 3, 5, 6, 8])
 def test_planes(lr, orc, e, k):
-    for batch, p in (([37], 16448 // e), ([1201], 1024 // e), ([3, 5], 65552 // e)):
+    for batch, p in (([37], 16448 // e), ([1201], 1024 // e), ([301], 576), ([301], 1024), ([3, 5], 65552 // e)):
         if len(batch) == 1:
             check(lr, orc, e, batch + [k, p], [0, 2, 1])
             check(lr, orc, e, batch + [p, k], [0, 2, 1])
