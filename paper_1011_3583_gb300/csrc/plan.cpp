@@ -32,7 +32,6 @@ constexpr int64_t kRunMinBytes = 128;     // cells this large are copied as runs
 constexpr int64_t kRunUnitBytes = 32768;  // payload of one runs work unit
 constexpr uint64_t kReorderL2MinBytes = uint64_t(128) << 20;  // reorder sources this large use L2 passes
 constexpr uint64_t kMaxUnits = 0xFFFFFFFFull;
-constexpr uint64_t kGatherStepMax = uint64_t(1) << 23;  // index sequences cut into single steps
 constexpr uint64_t kSpanMinCells = uint64_t(3) << 18;  // smaller thin-plane ops stay strided copies
 constexpr int64_t kPlaneMinCells = 576;  // shorter planes are no interlaces: see plan_planes()
 constexpr uint64_t kSpanLutCells = uint64_t(12) << 20; // thin planes whose spans need a table: see span_thin()
@@ -919,6 +918,30 @@ rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int 
     return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err, what);
 }
 
+// Groups of four elements per thread in a unit of an index gather or scatter of
+// n elements of one W-byte word (vec: the body of 16-byte index loads, which
+// holds two groups in flight).  One up to 2^23 elements and two beyond: with
+// eight, 3M elements were 367 CTAs for 152 SMs (us at one, two, four, eight:
+// 3,000,017 x 8 B random gather 17.6, 17.4, 20.3, 20.7, 65,536 x 4 B 2.3, 2.7,
+// 3.7, 5.2; 16M x 4 B 70.0, 68.3, 69.5, 70.5).  Where that is not enough work
+// for a CTA, or too much for an SM:
+// - 1- and 2-byte elements in local order read 4 to 8 KB a unit of 1024: 8M x
+//   1 B in shuffled blocks 9.7, 6.4, 6.0, 6.6, 40M 44.7, 33.5, 31.8, 33.2, 40M
+//   x 2 B 73.6, 59.5, 57.4, 58.2 (also by 64-bit indices: 162, 156, 153, 158);
+//   in random order the four are within 1 % from 3M on, below it one is ahead
+//   (1.5M x 1 B 7.3, 9.4).
+// - scatters of 8-byte elements write quarters of 32-byte sectors, which an SM
+//   joins only while one CTA does it: a CTA per SM as long as eight groups last
+//   (600,000 in shuffled blocks 5.0, 3.6, 2.9 (four), 4.3, 1.05M 6.0, 8.5, 5.8,
+//   4.4; in random order 5.4, 4.5, 4.7, 6.8 and 7.0, 9.2, 7.2, 7.0).
+static uint32_t gather_groups(uint64_t n, uint32_t W, bool vec, bool scatter)
+{
+    const uint64_t unit = uint64_t(kThreads) * 4, sms = 152;
+    if (vec && scatter && W == 8 && n <= 8 * unit * sms) return uint32_t((n + unit * sms - 1) / (unit * sms));
+    if (n > uint64_t(1) << 23) return W == 2 || (vec && W == 1) ? 4 : 2;
+    return vec && W <= 2 && n > uint64_t(5) << 19 ? 2 : 1;
+}
+
 rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_t n, size_t elem_bytes,
                           OpDesc &op, std::string &err, int idx_bytes, bool scatter)
 {
@@ -952,13 +975,7 @@ rearr_status plan_reorder(void *dst, const void *src, const uint32_t *idx, size_
     // the contiguous side (dst of a gather, src of a scatter) in groups of 4
     const uintptr_t contiguous = scatter ? sa : da;
     g.vec = (g.c == 1 && idx_bytes == 4 && ia % 16 == 0 && contiguous % uint64_t(std::min(16, 4 * W)) == 0) ? 1u : 0u;
-    // Units of one step of the body (four elements per thread) up to
-    // kGatherStepMax elements, of two beyond: with eight steps a unit, 3M
-    // elements were 367 CTAs for 152 SMs.  3,000,017 x 8 B random gather 23.9
-    // -> 20.5 us, 4M x 16 B 57 -> 42, 65,536 x 4 B 5.1 -> 3.5, scatter of
-    // 3,000,017 x 4 B 19.8 -> 16.4; at 16M x 4 B one step 78.0, two 75.5,
-    // four 76.6, eight 78.0 us.
-    g.unit_elems = uint32_t(kThreads) * (n <= kGatherStepMax ? 4 : 8);
+    g.unit_elems = uint32_t(kThreads) * 4 * gather_groups(n, uint32_t(W), g.vec != 0, scatter);
     op.units = (uint64_t(n) + g.unit_elems - 1) / g.unit_elems;
     // Sources much larger than the L2 go through the bucketed passes (which
     // fall back to this direct gather on the device if the indices turn out
