@@ -343,9 +343,13 @@ __device__ __forceinline__ bool edge_box(const StencilArgs &a, int64_t by, int64
 
 // Programmatic dependent launch: nothing of the payload is touched before the
 // kernel ahead on the stream is complete; the next one may then be launched
-// and fills the SMs as this one's last wave thins out.  Sweeps back to back,
-// 4096^2: order II 24.8 -> 22.7 us, clamped 28.1 -> 26.2; 4094^2 40.0 -> 37.7;
-// 8192^2 80.3 -> 78.2.
+// and fills the SMs as this one's last wave thins out.  Sweeps back to back on
+// a stream, us without and with it: 512^2 4.1, 2.8; 2048^2 order II 8.2, 5.8;
+// 4096^2 24.5, 22.0, clamped 27.2, 25.7; 4094^2 39.6, 37.1; 8192^2 80.1, 77.6 (a
+// sweep with no kernel ahead of it gains nothing).  Sweeps in a captured graph
+// follow each other closely as it is, and grids of the L2's size lose by it
+// there (2000 x 1600 order II 4.4, 5.1, clamped 8.2, 8.9; 900 x 2816 box 2
+// clamped 9.1, 10.9): launches under capture go without.
 __device__ __forceinline__ void pdl_enter()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -427,9 +431,12 @@ cudaError_t launch_one(const StencilPlan &pl, const CUtensorMap &m, cudaStream_t
     cfg.blockDim = dim3(kStencilThreads);
     cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = s;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = capture == cudaStreamCaptureStatusNone;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (pl.a.tma) return cudaLaunchKernelEx(&cfg, k_stencil_tma<R, BODY>, pl.a, m);

@@ -230,6 +230,37 @@ def test_table4_grid_4096(lr, orc, order):
                      ("4096", order, boundary))
 
 
+@pytest.mark.parametrize("captured", [False, True])
+def test_sweeps_follow_each_other(lr, orc, captured):
+    """Sweeps that read what the one ahead wrote, launched back to back on a
+    stream and captured in a graph, on grids of less than a wave, of a few
+    waves and without 16-byte rows."""
+    import torch
+    taps = f32_taps(fd_laplacian(1))
+    for ny, nx in ((70, 130), (781, 2816), (600, 1003)):
+        a, b = to_dev(grid(ny, ny, nx)), DevBuf(ny * nx * 4, fill=0)
+
+        def sweeps(stream):
+            for _ in range(3):
+                lr.stencil2d(b.ptr, a.ptr, ny, nx, taps, 1, stream)
+                lr.stencil2d(a.ptr, b.ptr, ny, nx, taps, 1, stream)
+
+        st = torch.cuda.Stream()
+        st.wait_stream(torch.cuda.current_stream())
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=st):
+                sweeps(torch.cuda.current_stream())
+            graph.replay()
+        else:
+            sweeps(st)
+        sync()
+        src = grid(ny, ny, nx)
+        for _ in range(6):  # sweep by sweep, so that each bound is that of one sweep
+            src = run(lr, src, taps, 1)
+        assert np.array_equal(a.download().view(np.float32).reshape(ny, nx), src), (ny, nx)
+
+
 @pytest.mark.parametrize("order", [1, 4])
 def test_large_grid_sampled_rows(lr, orc, order):
     """A 16384 x 16384 grid (1 GiB each way), rows sampled at the edges, at
