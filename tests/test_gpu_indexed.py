@@ -46,6 +46,21 @@ def test_scatter_permutation(lr, orc, e):
         assert np.array_equal(got, orc.indexed(src, p64, e, scatter=False)), (n, e, "gather64")
 
 
+# on either side of the lines between units of one, two and four groups of
+# elements a thread, and of an 8-byte scatter's CTA per SM (one to eight groups)
+@pytest.mark.parametrize("e,n", [(1, 5 << 19), (1, (5 << 19) + 1), (2, (1 << 23) + 3), (4, 1 << 23), (4, (1 << 23) + 5),
+                                 (8, 152 * 1024), (8, 152 * 1024 + 1), (8, 700_001), (8, 8 * 152 * 1024),
+                                 (8, 8 * 152 * 1024 + 2)])
+def test_unit_sizes(lr, orc, e, n):
+    src, p = synth.random_elements(e, n, e), synth.random_permutation(n % 31, n)
+    for wide in (False, True):
+        idx = p.astype(np.uint64) if wide else p
+        got = run(lr, lr.scatter64 if wide else lr.scatter, src, idx, e, n, fill=0)
+        assert np.array_equal(got, orc.indexed(src, idx, e, scatter=True)), (e, n, wide)
+        got = run(lr, lr.reorder64 if wide else lr.reorder, src, idx, e, n, fill=0)
+        assert np.array_equal(got, orc.indexed(src, idx, e, scatter=False)), (e, n, wide)
+
+
 def test_scatter_unaligned(lr, orc):
     n = 5003
     for e, so, do, io in [(4, 4, 0, 4), (4, 0, 8, 0), (8, 8, 4, 8), (2, 2, 6, 12), (1, 1, 3, 4)]:
