@@ -90,6 +90,54 @@ def test_crowded(lr, e):
     check(lr, e, synth.random_indices(5, n, n // 2).astype(np.uint64))
 
 
+@pytest.mark.parametrize("e", [4, 8])
+@pytest.mark.parametrize("step", [17, 31, 1001])
+def test_strides(lr, e, step):
+    """Orders of a fixed stride, where a warp's indices rank in one list."""
+    n = MIN // e + 4097
+    while np.gcd(step, n) != 1:
+        step += 1
+    check(lr, e, (np.arange(n, dtype=np.uint64) * np.uint64(step) % np.uint64(n)).astype(np.uint32))
+
+
+@pytest.mark.parametrize("form", ["scatter", "reorder"])
+def test_capture(lr, form):
+    """The whole pass sequence captured in a graph and replayed on sequences that
+    take each of its branches: random, local, crowded."""
+    import torch
+    n = MIN // 4 + 77
+    s, ix, d = DevBuf(n * 4, fill=0), DevBuf(n * 4, fill=0), DevBuf(n * 4, fill=0)
+    call = getattr(lr, form)
+    call(d.ptr, s.ptr, ix.ptr, n, 4)  # set-up outside the capture
+    sync()
+    st = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        call(d.ptr, s.ptr, ix.ptr, n, 4, torch.cuda.current_stream())
+    blocks = (synth.random_permutation(5, n // 4096)[:, None].astype(np.uint32) * np.uint32(4096)
+              + np.arange(4096, dtype=np.uint32)).reshape(-1)
+    local = np.concatenate([blocks, np.arange(blocks.size, n, dtype=np.uint32)])
+    for seed, idx in enumerate((synth.random_permutation(6, n), local, synth.random_indices(7, n, n // 3),
+                                synth.random_permutation(8, n))):
+        src = synth.random_elements(seed, n, 4)
+        s.upload(src)
+        ix.upload(idx)
+        graph.replay()
+        sync()
+        got, src = d.download().view(np.uint32), src.view(np.uint32)
+        if form == "reorder":
+            assert np.array_equal(got, src[idx]), seed
+        elif np.unique(idx).size == n:
+            assert np.array_equal(got[idx], src), seed
+        else:  # each written element carries a source that names it (values are unique enough to look up)
+            key = (idx.astype(np.uint64) << np.uint64(32)) | src
+            key.sort()
+            at = np.unique(idx)
+            want = (at.astype(np.uint64) << np.uint64(32)) | got[at]
+            pos = np.searchsorted(key, want)
+            assert np.array_equal(key[np.minimum(pos, n - 1)], want), seed
+
+
 def test_two_threads(lr):
     """Calls of different sizes (so of different shared-memory needs) from two
     threads at a time."""
