@@ -157,7 +157,7 @@ static void fill_tile_common(TileDesc &t, const std::vector<Axis> &ax, int p, in
 {
     const int R = int(ax.size());
     // Output strides (cells) of the canonical output axes, row-major.
-    std::vector<int64_t> os(R);
+    int64_t os[kMaxRank];
     os[R - 1] = 1;
     for (int i = R - 2; i >= 0; --i) os[i] = os[i + 1] * ax[i + 1].extent;
     const int64_t DA = ax[p].extent, DB = ax[R - 1].extent;
@@ -384,6 +384,7 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     const uint64_t bytes = total * elem_bytes;
     // Axes with extent > 1, merged where adjacent and in order.
     std::vector<Axis> ax;
+    ax.reserve(in_axes.size());
     for (const Axis &cur : in_axes) {
         if (cur.extent == 1) continue;
         if (!ax.empty() && ax.back().stride == cur.stride * cur.extent) {
@@ -731,7 +732,7 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     if (pl.use_planes) return REARR_OK;
     if (span_tile) {
         pl.use_span = plan_span(ax, cell, d, src, pl.span);
-    } else if (thin && (cell < 4 || (cell == 4 && ax.back().extent >= 32))) {
+    } else if (thin && (cell < 4 || (cell == 4 && ax.back().extent >= 32 && ax.back().stride >= 16))) {
         const bool lut = cell < 4 && n_cells >= kSpanLutCells;
         pl.use_span = plan_span(ax, cell, d, src, pl.span, true, lut) && span_thin(pl.span, lut);
     }
@@ -817,10 +818,18 @@ bool plan_planes(const std::vector<Axis> &ax, int64_t E, char *dst, const char *
     return true;
 }
 
+// The parts of a plan that its flags do not cover, zeroed.
+static void clear(PermPlan &pl)
+{
+    std::memset(&pl.info, 0, sizeof(pl.info));
+    std::memset(&pl.op, 0, sizeof(pl.op));
+    pl.use_planes = pl.use_span = pl.use_batch_span = false;
+}
+
 rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int rank, const int64_t *dims,
                           const int *perm, PermPlan &pl, std::string &err, PlanFor what)
 {
-    std::memset(&pl, 0, sizeof(pl));
+    clear(pl);
     rearr_permute_info &info = pl.info;
     info.plane_a = -1;
     info.wide_a = info.wide_b = -1;
@@ -859,6 +868,7 @@ rearr_status plan_permute(void *dst, const void *src, size_t elem_bytes, int ran
     s[rank - 1] = int64_t(elem_bytes);
     for (int i = rank - 2; i >= 0; --i) s[i] = s[i + 1] * dims[i + 1];
     std::vector<Axis> ax;
+    ax.reserve(size_t(rank));
     for (int i = 0; i < rank; ++i) ax.push_back(Axis{dims[perm[i]], s[perm[i]]});
     return plan_axes(dst, static_cast<const char *>(src), elem_bytes, ax, total, pl, err, what);
 }
@@ -867,7 +877,7 @@ rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int 
                              int rank_out, const int *order, const int64_t *base, const int64_t *range,
                              PermPlan &pl, std::string &err, PlanFor what)
 {
-    std::memset(&pl, 0, sizeof(pl));
+    clear(pl);
     pl.info.plane_a = -1;
     pl.info.wide_a = pl.info.wide_b = -1;
     if (elem_bytes == 0) { err = "elem_bytes must be >= 1"; return REARR_EINVAL; }
@@ -914,6 +924,7 @@ rearr_status plan_reorder_nm(void *dst, const void *src, size_t elem_bytes, int 
     int64_t off = 0;
     for (int a = 0; a < rank_in; ++a) off += base[a] * s[a];
     std::vector<Axis> ax;
+    ax.reserve(size_t(rank_out));
     for (int i = 0; i < rank_out; ++i) ax.push_back(Axis{range[order[i]], s[order[i]]});
     return plan_axes(dst, static_cast<const char *>(src) + off, elem_bytes, ax, total, pl, err, what);
 }
