@@ -202,41 +202,63 @@ __device__ __forceinline__ void load_tile(const L2Reorder &p, uint32_t i0, uint3
 }
 
 // Bucket starts and scatter units from the bucket sizes, by one CTA (the last
-// one of the histogram pass to finish).
-__device__ __forceinline__ void scan_buckets(const L2Reorder &p, uint32_t *warp_sums, uint32_t *total)
+// one of the histogram pass to finish).  Eight buckets a thread and round, a
+// warp's apart by kThreads: loads and stores of a round are in flight together
+// and coalesced, and one warp scans the warps' sums for all of them.
+constexpr int kScanPer = 8;
+
+__device__ __forceinline__ void scan_buckets(const L2Reorder &p, uint32_t (&sums)[kScanPer * kWarps + 1])
 {
-    const uint32_t nb = p.C * p.D;
-    auto scan = [&](uint32_t v) {
-        const uint32_t e = cta_scan<kThreads>(v, warp_sums);
-        if (threadIdx.x == kThreads - 1) *total = e + v;
-        __syncthreads();
-        return e;
+    static_assert(kScanPer * kWarps == 64, "two sums a lane");
+    const uint32_t nb = p.C * p.D, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto scan = [&](auto size, auto store) {
+        uint32_t carry = 0;
+        for (uint32_t b0 = 0; b0 < nb; b0 += kThreads * kScanPer) {
+            const uint32_t b = b0 + threadIdx.x;
+            uint32_t v[kScanPer], x[kScanPer];
+#pragma unroll
+            for (int j = 0; j < kScanPer; ++j) v[j] = b + j * kThreads < nb ? size(b + j * kThreads) : 0u;
+#pragma unroll
+            for (int j = 0; j < kScanPer; ++j) {
+                x[j] = v[j];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, x[j], o);
+                    if (lane >= o) x[j] += y;
+                }
+                if (lane == 31) sums[j * kWarps + w] = x[j];
+            }
+            __syncthreads();
+            if (w == 0) {
+                const uint32_t s0 = sums[2 * lane], s1 = sums[2 * lane + 1];
+                uint32_t y = s0 + s1;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+                    if (lane >= o) y += z;
+                }
+                sums[2 * lane] = y - s0 - s1;
+                sums[2 * lane + 1] = y - s1;
+                if (lane == 31) sums[kScanPer * kWarps] = y;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kScanPer; ++j)
+                if (b + j * kThreads < nb) store(b + j * kThreads, carry + sums[j * kWarps + w] + x[j] - v[j]);
+            carry += sums[kScanPer * kWarps];
+            __syncthreads();
+        }
+        return carry;
     };
-    uint32_t carry = 0;
-    for (uint32_t b0 = 0; b0 < nb; b0 += kThreads) {  // bucket starts, c-major
-        const uint32_t b = b0 + threadIdx.x;
-        const uint32_t e = scan(b < nb ? __ldcg(p.hist + b) : 0u);
-        if (b < nb) {
-            p.base[b] = carry + e;
-            p.cursor[b] = carry + e;
-        }
-        carry += *total;
-        __syncthreads();
-    }
-    carry = 0;
-    for (uint32_t s0 = 0; s0 < nb; s0 += kThreads) {  // scatter units, d-major (s = d*C + c)
-        const uint32_t s = s0 + threadIdx.x;
-        uint32_t v = 0;
-        if (s < nb) {
+    scan([&](uint32_t b) { return __ldcg(p.hist + b); },  // bucket starts, c-major
+         [&](uint32_t b, uint32_t at) { p.base[b] = p.cursor[b] = at; });
+    const uint32_t units = scan(  // scatter units, d-major (s = d*C + c)
+        [&](uint32_t s) {
             const uint32_t d = s / p.C, c = s - d * p.C;
-            v = (__ldcg(p.hist + c * p.D + d) + kTile - 1) / kTile;
-        }
-        const uint32_t e = scan(v);
-        if (s < nb) p.uprefix[s] = carry + e;
-        carry += *total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) p.uprefix[nb] = carry;
+            return (__ldcg(p.hist + c * p.D + d) + kTile - 1) / kTile;
+        },
+        [&](uint32_t s, uint32_t at) { p.uprefix[s] = at; });
+    if (threadIdx.x == 0) p.uprefix[nb] = units;
 }
 
 // Each CTA walks a contiguous range of tiles with per-warp shared counters
@@ -299,7 +321,7 @@ __global__ void __launch_bounds__(kThreads) k_l2_hist(const L2Reorder p, uint32_
         if (c < p.C && row[j]) atomicAdd(&p.rowtot[c], row[j]);
     }
     // The last CTA to get here has every count behind it.
-    __shared__ uint32_t warp_sums[32], total;
+    __shared__ uint32_t sums[kScanPer * kWarps + 1];
     __shared__ bool last;
     __threadfence();
     __syncthreads();
@@ -307,7 +329,7 @@ __global__ void __launch_bounds__(kThreads) k_l2_hist(const L2Reorder p, uint32_
     __syncthreads();
     if (last) {
         __threadfence();
-        scan_buckets(p, warp_sums, &total);
+        scan_buckets(p, sums);
     }
 }
 
