@@ -373,6 +373,14 @@ rearr_status rearr_plan_stats(const rearr_plan *plan, int64_t *n_ops, int64_t *n
  * element, and classifies the op (the offset and stride computation and the 2-D
  * plane of Sec. III.B: the plane of the input's fastest and the output's
  * fastest dimension).
+ *
+ * The class and its geometry are those of the op's kernel in a work list: what
+ * rearr_batch_noalloc, the server, small captured plans and a pipeline's direct
+ * ops run.  A single call may run another kernel in its place, with the same
+ * result: interlaces for a permute of up to 8 long dense planes on 16-byte
+ * boundaries, a span copy (contiguous spans of both sides by way of shared
+ * memory) for a tile without 16-byte loads or with few of its cells used, and
+ * for many large thin planes.  Large captured plans run span copies too.
  * ------------------------------------------------------------------------- */
 typedef enum {
     REARR_KIND_NOOP = 0,        /* zero elements                                */

@@ -24,7 +24,7 @@ struct Axis {
 enum class PlanFor { kCall, kBatch, kOp };
 
 struct PermPlan {
-    rearr_permute_info info;  // what rearr_permute_describe reports
+    rearr_permute_info info;  // what rearr_permute_describe reports: op and its geometry
     OpDesc op;                // descriptor of the work-list body
     // kCall: what runs instead, if there is one: interlaces of a few planes, or
     // a span copy.
