@@ -157,7 +157,9 @@ def test_large_batch(lr, orc):
             op["src"] = [synth.random_elements(1000 * replay + i + 7 * j, op["n"], op["e"]) for j in range(len(op["in"]))]
             for b, a in zip(op["in"], op["src"]):
                 b.upload(a)
+        before = lr.launch_count()
         plan.run()
+        assert lr.launch_count() - before == 3  # split: gathers, the rest, span copies
         sync()
         for op in ops:
             e, n, src = op["e"], op["n"], op["src"]
@@ -172,3 +174,32 @@ def test_large_batch(lr, orc):
             else:
                 want = orc.interlace(src, n, e)
             assert np.array_equal(op["out"].download(), want), (replay, op["kind"], e, n, op.get("dims"))
+
+
+@pytest.mark.parametrize("others,kernels", [(0, 1), (3, 2)])
+def test_split_without_spans(lr, orc, others, kernels):
+    """Plans that are split but leave a kernel without ops: index gathers alone,
+    and with interlaces and full tiles beside them."""
+    plan = lr.Plan()
+    want = []
+    for i in range(21):  # 2048 units each
+        n = (1 << 22) - i
+        src, idx = synth.random_elements(i, n, 1), synth.random_permutation(i, n)
+        d = DevBuf(n, fill=0x55)
+        bufs = (to_dev(src), to_dev(idx), d)
+        plan.add_reorder(d.ptr, bufs[0].ptr, bufs[1].ptr, n, 1)
+        want.append((bufs, d, orc.reorder(src, idx, 1)))
+    for i in range(others):
+        dims, perm = ([128, 64, 256], [2, 0, 1]) if i % 2 else ([256, 512], [1, 0])
+        n = int(np.prod(dims))
+        src = synth.random_elements(50 + i, n, 4)
+        s, d = to_dev(src), DevBuf(n * 4, fill=0x55)
+        plan.add_permute(d.ptr, s.ptr, 4, dims, perm)
+        want.append((s, d, orc.permute(src, 4, dims, perm)))
+    plan.finalize()
+    before = lr.launch_count()
+    plan.run()
+    assert lr.launch_count() - before == kernels
+    sync()
+    for _, d, w in want:
+        assert np.array_equal(d.download(), w)
