@@ -7,7 +7,7 @@
 // 6 CTAs per SM), the alignment being carried into shared memory, and output
 // spans are put together from shared memory in 4-byte words (whole cells from
 // 4 bytes up) so that a warp writes 128 contiguous bytes.  Spans' offsets come
-// from tables built once per CTA; a CTA's units are kThreads apart.
+// from tables built once per CTA; a CTA's units are gridDim.x apart.
 // Bounds: DRAM for cells of 4 bytes and more (251 x 333 x 517 fp32 in order
 // 2,0,1: 150 us as narrow tiles, 68 us, 5.1 TB/s; 8-byte cells 5.8 TB/s),
 // instruction issue and shared-memory reads (one per cell) below (2-byte 52 us,
@@ -28,8 +28,8 @@ constexpr int kSpanCtas = 6;  // resident CTAs per SM (about 40 registers a thre
 template <int E, bool LUT>
 __global__ void __launch_bounds__(kThreads, kSpanCtas) k_span(const __grid_constant__ SpanDesc d)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SpanUnit unit;
+    extern __shared__ __align__(32) unsigned char smem[];
+    __shared__ SpanUnit unit[2];
     // The tables read no global memory, so they are built before the wait for
     // the kernel ahead on the stream.
     span_units<E, LUT>(d, blockIdx.x, d.units, gridDim.x, smem, unit, [] {
@@ -44,7 +44,8 @@ __global__ void __launch_bounds__(kThreads, kSpanCtas) k_span(const __grid_const
 constexpr uint64_t kBatchSpanGrab = 16;
 
 template <int E, bool LUT>
-__device__ __noinline__ void span_range(const SpanDesc &d, uint32_t u0, uint32_t u1, unsigned char *smem, SpanUnit &unit)
+__device__ __noinline__ void span_range(const SpanDesc &d, uint32_t u0, uint32_t u1, unsigned char *smem,
+                                        SpanUnit (&unit)[2])
 {
     span_units<E, LUT>(d, u0, u1, 1, smem, unit, [] {});
 }
@@ -53,8 +54,8 @@ __global__ void __launch_bounds__(kThreads, kSpanCtas) k_batch_span(const SpanDe
                                                                    const uint64_t *__restrict__ prefix, int n,
                                                                    unsigned long long *counter, uint32_t grab)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SpanUnit unit;
+    extern __shared__ __align__(32) unsigned char smem[];
+    __shared__ SpanUnit unit[2];
     __shared__ SpanDesc d;
     __shared__ unsigned long long s_start;
     const uint64_t total = prefix[n];
