@@ -449,9 +449,10 @@ rearr_status rearr_tuning_load(const char *path);
  *   rearr_launch_count : number of kernels this library has launched in this
  *                        process (graph replays count the kernels they run).
  *   rearr_selftest_host: host-only checks of the plan compiler's integer
- *                        helpers, and box plans of pseudo-random permutes run
- *                        on the host against the permute written out;
- *                        returns REARR_OK when they all pass.
+ *                        helpers, routes and scatter geometry; box, span and
+ *                        interlace plans of pseudo-random permutes run on the
+ *                        host against the permute written out; returns
+ *                        REARR_OK when they all pass.
  * ------------------------------------------------------------------------- */
 rearr_status rearr_memcpy_d2d(void *dst, const void *src, size_t bytes, rearr_stream_t stream);
 uint64_t rearr_launch_count(void);

@@ -85,11 +85,11 @@ struct ListGeometry {
 // n elements of W bytes; chunks as large as shared memory takes, evened out
 // over the sms SMs where each places only a few; scratch from byte `start` to
 // byte `limit` of the call's.  Measured against the bucketed passes (random
-// permutations, us): 2^25 x 4 B 422 -> 272, 2^26 796 -> 559, 10^8 1167 -> 881,
-// 2^27 1538 -> 1290, 2^28 3058 -> 3489; 2^24 x 8 B 302 -> 239, 2^25 549 -> 471,
-// 2^26 1056 -> 1127; 2^23 x 16 B 249 -> 240, 2^25 895 -> 1148: tiles' segments
-// have to be long enough for their list writes to fill sectors, and 16-byte
-// elements (tiles of 8192) gain nothing.
+// permutations, us): 2^25 x 4 B 424 -> 260, 2^26 801 -> 529, 10^8 1160 -> 789,
+// 2^27 1537 -> 1130; 2^24 x 8 B 302 -> 212, 2^25 553 -> 418.  Left out, as first
+// built: 2^28 x 4 B 3058 -> 3489, 2^26 x 8 B 1056 -> 1127, 2^23 x 16 B 249 -> 240,
+// 2^25 x 16 B 895 -> 1148: tiles' segments have to be long enough for their list
+// writes to fill sectors, and 16-byte elements (tiles of 8192) gain nothing.
 inline ListGeometry list_geometry(uint64_t n, uint32_t W, uint32_t sms, size_t start, size_t limit)
 {
     ListGeometry g{};

@@ -14,11 +14,11 @@
 //           marked ones out.
 // 24 bytes of DRAM traffic per 4-byte element (idx 4, its second read in the
 // L2; src 4, list 6 + 6, dst 4) and two kernels; the passes this replaces end
-// in random stores (0.69 per clock per SM at most).  10^8 x 4 B random: 1167 ->
-// 905 us, lists 594 us (shared-memory wavefronts, 60 % of the pipe's cycles:
-// ranking and placing are random accesses; one CTA of 1024 threads per SM, as
-// tiles half as large at two CTAs halved the segments and took 1114 us in
-// all), place 247 us (3.8 TB/s).  An element whose list is full is stored at
+// in random stores (0.69 per clock per SM at most).  10^8 x 4 B random: 1160 ->
+// 789 us, of which about 3/4 lists (shared-memory wavefronts, 60 % of the pipe's
+// cycles: ranking and placing are random accesses; one CTA of 1024 threads per
+// SM: before lists had their present length, tiles half as large at two CTAs
+// halved the segments and took 1114 us in all instead of 905), 1/4 place.  An element whose list is full is stored at
 // once to its place in the destination (which of several elements of one
 // destination stays is unspecified).  Where the sample says that many would be,
 // the lists set a flag on which the place pass returns and the bucketed passes

@@ -157,9 +157,8 @@ __device__ __forceinline__ typename Word<E * V>::T span_word(const unsigned char
 // 32-byte boundary (two chunks of a sector that land in one 32-byte line of
 // shared memory are one request: 16 bytes off, 251 x 333 x 517 of 8 bytes in
 // order 2,0,1 read 33.0 M sectors from the L2 instead of 22.2 M, 130 against 119
-// us) and
-// unit[] in shared memory.  start(): called once the tables stand and before
-// anything of the payload is read.  Ends with a barrier.
+// us), and unit[] in shared memory.  start(): called once the tables stand and
+// before anything of the payload is read.  Ends with a barrier.
 template <int E, bool LUT, class Start>
 __device__ __forceinline__ void span_units(const SpanDesc &d, uint32_t u0, uint32_t u1, uint32_t u_step,
                                            unsigned char *smem, SpanUnit (&unit)[2], Start start)
