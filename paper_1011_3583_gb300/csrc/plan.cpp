@@ -356,6 +356,31 @@ static bool plan_box(const std::vector<Axis> &ax, int64_t E, uintptr_t da, uintp
     return true;
 }
 
+// Output spans of 1- and 2-byte cells over several axes, the first of them across
+// input spans of a stride that is a multiple of 16 bytes: how many lanes of a
+// store read different words of one bank (lanes are 4 / E cells apart, so they
+// meet n0 / gcd(n0, 4 / E) of the n0 input spans); 1 for other plans.
+static uint32_t span_bank_lanes(const SpanDesc &d)
+{
+    if (!d.lut || d.fixed || d.E > 2 || d.ch_sm[0] % 16 != 0) return 1;
+    uint32_t g = 4 / d.E;
+    while (d.ch_ext[0].d % g != 0) g /= 2;
+    const uint32_t spans = std::min(32u, d.ch_ext[0].d / g);
+    uint32_t banks = 32;
+    for (uint32_t words = g * d.ch_sm[0] / 4; banks > 1 && words % 2 == 0; words /= 2) banks /= 2;
+    return spans / std::min(banks, spans);
+}
+
+// From this many on the strided copy is faster (us, strided against spans).  In
+// a call of its own, last two axes swapped: with four lanes 200 x 16 x 4096
+// bytes 13.8, 14.2; eight 200 x 32 x 4096 21.6, 33.5; twelve 512 x 48 x 512
+// 13.2, 23.8, of 2 bytes 15.6, 21.6.  In a batch of 800 MB the span units run in
+// one kernel with nothing beside them: with eight 64 x 32 x 512 bytes 1024, 970,
+// 64 x 512 x 8 of 2 bytes 1595, 533; twelve 64 x 48 x 512 bytes 810, 1309, of 2
+// bytes 591, 629.
+constexpr uint32_t kSpanBankLanes = 8;
+constexpr uint32_t kSpanBankLanesBatch = 12;
+
 // Whether a thin plane's span copy beats its strided copy (us, strided against
 // span).  Output spans over several axes take their offsets from a table and
 // their words one by one: that pays where every span fits one pass of the lanes
@@ -364,14 +389,17 @@ static bool plan_box(const std::vector<Axis> &ax, int64_t E, uintptr_t da, uintp
 // x 597 7.0, 8.0; 2 bytes: 34 x 3 x 372 x 511 24.4, 17.6, but 36 x 6 x 557 x 35
 // 6.8, 9.5; 4 bytes: 12 x 2 x 363 x 273 4.3, 6.0, 57 x 4 x 151 x 829 39.2, 39.4).
 // A span of 32 words or more whose words all lie in one bank takes a cycle a
-// lane (4 x 1168 x 2416 bytes reversed 43.7, 51.5).  Taking every third 4-byte
-// cell apart is near the copy rate either way (1817 x 1490 x 3 10.3, 12.4),
-// every fourth is not (28 x 31 x 1218 x 4 11.1, 7.2).
+// lane (4 x 1168 x 2416 bytes reversed 43.7, 51.5; 64 x 512 x 32 of 2 bytes 6.2,
+// 8.0; single bytes along one axis still gain, 512 x 512 x 32 41.5, 34.7).
+// Taking every third 4-byte cell apart is near the copy rate either way
+// (1817 x 1490 x 3 10.3, 12.4), every fourth is not (28 x 31 x 1218 x 4 11.1,
+// 7.2).
 static bool span_thin(const SpanDesc &d, bool lut)
 {
-    if (d.lut && !d.fixed) return lut;
-    if (d.lut) return d.store_lanes.d < 32 || d.ch_sm[0] * (4 / d.E) % 128 != 0;
-    return d.E < 4 || d.ch_sm[0] >= 16;
+    if (d.lut && !d.fixed) return lut && span_bank_lanes(d) < kSpanBankLanes;
+    const bool one_bank = d.store_lanes.d >= 32 && d.ch_sm[0] * (4 / d.E) % 128 == 0;
+    if (one_bank && (d.lut || d.E == 2)) return false;
+    return d.lut || d.E < 4 || d.ch_sm[0] >= 16;
 }
 
 // Plans a gather of `total` elements of elem_bytes whose output axes are
@@ -725,7 +753,9 @@ static rearr_status plan_axes(void *dst, const char *src, size_t elem_bytes, con
     const bool thin = op.cls == OC_STRIDED && n_cells >= kSpanMinCells;
     char *d = static_cast<char *>(dst);
     if (what == PlanFor::kBatch) {
-        pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || span_tile) && plan_span(ax, cell, d, src, pl.span, false);
+        pl.use_batch_span = cell <= 8 && (op.cls == OC_STRIDED || span_tile) &&
+                            plan_span(ax, cell, d, src, pl.span, false) &&
+                            span_bank_lanes(pl.span) < kSpanBankLanesBatch;
         return REARR_OK;
     }
     pl.use_planes = (thin || narrow || (tile && 3 * n_cells < 2 * held)) && plan_planes(ax, cell, d, src, pl.planes_op);
@@ -1340,6 +1370,8 @@ static bool selftest_routes(std::string &err)
         {0, 2, 4, {36, 6, 557, 35}, {0, 2, 3, 1}},
         {0, 4, 4, {12, 2, 363, 273}, {0, 2, 3, 1}},   // 4-byte cells
         {0, 1, 3, {4, 1168, 2416}, {2, 1, 0}},        // words of a span in one bank
+        {0, 2, 3, {64, 512, 32}, {0, 2, 1}},
+        {0, 1, 3, {512, 48, 512}, {0, 2, 1}},         // of many spans
         {0, 4, 3, {20480, 2, 128}, {0, 2, 1}},        // short planes
         {0, 8, 3, {6826, 64, 6}, {0, 2, 1}},
         {2, 4, 3, {2048, 3, 1024}, {0, 2, 1}},        // long ones
